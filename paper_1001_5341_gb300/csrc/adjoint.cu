@@ -50,7 +50,7 @@ __global__ void k_adj_probes(Grid g, float *E, Probes p, const float *__restrict
 }
 
 // dL/dqbar of step n: the sum over the footprint edges of mu_Ez times the E
-// increment per unit qbar (the deposit pattern of source_term without qbar).
+// increment per unit qbar (the deposit pattern of source_amp without qbar).
 constexpr int ADJ_THREADS = 256;
 
 __global__ void k_adj_source(Grid g, const float *__restrict__ E, Source s, SourceStep w, double *__restrict__ out) {
@@ -164,11 +164,12 @@ __global__ void __launch_bounds__(256) k_adj_h(Grid g, const float *__restrict__
     cell_h(g, Et, Hin, Hout, pml, kH, i, j, k);
 }
 
-__global__ void __launch_bounds__(256) k_adj_e(Grid g, float *E, const float *__restrict__ H, Cpml pml, float kE,
-                                               Source src) {
+__global__ void __launch_bounds__(256) k_adj_e(Grid g, float *E, const float *__restrict__ H, Cpml pml, float kE) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
     if (i >= g.nx || j >= g.ny) return;
-    cell_e(g, E, H, E, pml, kE, src, 0, i, j, k);   // in place: each cell reads and writes only itself
+    Source none{};
+    const SourceStep empty = source_window(none, 0);
+    cell_e(g, E, H, E, pml, kE, none, empty, i, j, k);   // in place: each cell reads and writes only itself
 }
 
 __device__ __forceinline__ float hval(const Grid &g, const float *Hc, int i, int j, int k) {
@@ -218,12 +219,11 @@ void adj_field_step_mur(fdtd_ctx *h) {
     const float *in = h->fields[h->cur];
     float *out = h->fields[h->cur ^ 1];
     const float m = (float)h->mur_m;
-    Source none{};
     const Cpml pml = cpml_view(h);   // P = 0 on a Mur grid
     k_adj_mur_gather<<<dim3((g.nx + 1 + 127) / 128, g.ny + 1, g.nz + 1), 128, 0, h->stream>>>(g, in, out, m);
     const dim3 blk(32, 8, 1), grd((g.nx + 31) / 32, (g.ny + 7) / 8, g.nz);
     k_adj_h<<<grd, blk, 0, h->stream>>>(g, out, in + 3 * g.comp, out + 3 * g.comp, pml, (float)-h->kE);
-    k_adj_e<<<grd, blk, 0, h->stream>>>(g, out, out + 3 * g.comp, pml, (float)-h->kH, none);
+    k_adj_e<<<grd, blk, 0, h->stream>>>(g, out, out + 3 * g.comp, pml, (float)-h->kH);
     int amax = (g.nx > g.ny ? g.nx : g.ny) + 1;
     int bmax = (g.ny > g.nz ? g.ny : g.nz) + 1;
     if (g.nz + 1 > bmax) bmax = g.nz + 1;

@@ -195,10 +195,8 @@ __global__ void __launch_bounds__(NT, 1) k_batch(BArgs A) {
                 for (int w = tid; w < (int)(sizeof(vt::Args) / 8); w += NT) dst[w] = src[w];
             }
             __syncthreads();
-            if (tid == 0) {
-                s_a.ss = source_window(s_a.src, S.n + s);
-                s_a.flags = A.flags;
-            }
+            if (tid < 32 && vt::src_tile(s_a, item % S.tiles)) source_step_warp(s_a.src, S.n + s, &s_a.ss);
+            if (tid == 0) s_a.flags = A.flags;
             __syncthreads();
             const int ns = vt::tile_block<false>(s_a, *S.maps, item % S.tiles, item / S.tiles, smem_raw);
             vt::end_tile(smem_raw, ns);

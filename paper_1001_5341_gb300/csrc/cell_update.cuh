@@ -65,7 +65,7 @@ __device__ __forceinline__ void cell_h(const Grid &g, const float *__restrict__ 
 // Ein, Eout: Ex of sets cur / cur^1; Hnew: Hx of set cur^1.
 __device__ __forceinline__ void cell_e(const Grid &g, const float *__restrict__ Ein,
                                        const float *__restrict__ Hnew, float *__restrict__ Eout,
-                                       const Cpml &pml, float kE, const Source &src, long long n,
+                                       const Cpml &pml, float kE, const Source &src, const SourceStep &ss,
                                        int i, int j, int k) {
     const float *Hx = Hnew, *Hy = Hnew + g.comp, *Hz = Hnew + 2 * g.comp;
     long long c = gidx(g, i, j, k);
@@ -91,7 +91,7 @@ __device__ __forceinline__ void cell_e(const Grid &g, const float *__restrict__ 
         if (lx >= 0) cpml_inplace(pml.e[0][1] + psi_x(g, P, lx, j, k), pml.aE[0], pml.bE[0], i, dx);
         if (ly >= 0) cpml_inplace(pml.e[1][1] + psi_y(g, W, i, ly, k), pml.aE[1], pml.bE[1], j, dy);
         float e = Ein[2 * g.comp + c] + kE * (dx - dy);
-        if (src.active) e += source_term(src, i, j, k, n);
+        e += source_at(src, ss, i, j, k);
         Eout[2 * g.comp + c] = e;
     }
 }

@@ -287,6 +287,11 @@ int fdtd_set_shower(fdtd_t h, const double *q, int n_bins, double z0, double bin
     }
     TRY(h, cudaMemcpy(h->d_q, q, sizeof(double) * n_bins, cudaMemcpyHostToDevice));
     TRY(h, cudaMemcpy(h->d_w, w, sizeof(double) * nw, cudaMemcpyHostToDevice));
+    try {
+        h->h_q.assign(q, q + n_bins);
+    } catch (const std::bad_alloc &) {
+        return FDTD_ERR_OOM;
+    }
     Source &s = h->src;
     s.L = L; s.ic = ic; s.jc = jc;
     s.kmin = h->boundary == FDTD_CPML ? h->P : 0;

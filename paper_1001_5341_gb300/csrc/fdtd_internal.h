@@ -101,10 +101,15 @@ struct Source {
     const double *w;          // lateral weights (2L+1)^2
 };
 
-// window of planes whose Ez edges may carry the shower's current in step n
+// the shower's current of step n: the planes whose Ez edges carry it and, for
+// up to SRC_PLANES of them, the E increment per unit lateral weight on plane
+// kb + t (amp[t]; source_term.cuh)
+constexpr int SRC_PLANES = 8;
 struct SourceStep {
     long long n;
-    int klo, khi;
+    int klo, khi;             // planes that may carry current (empty: klo > khi)
+    int kb, tab;              // tab: amp covers the window, from plane kb
+    double amp[SRC_PLANES];
 };
 
 struct Probes {
@@ -153,6 +158,7 @@ struct fdtd_ctx {
     // source
     double *d_q;
     double *d_w;
+    std::vector<double> h_q;  // the charge table, for the per-launch source amplitudes
     fdtd::Source src;
 
     // detectors

@@ -31,15 +31,15 @@ __global__ void __launch_bounds__(256) k_update_h(Grid g, const float *__restric
     cell_h(g, Ein, Hin, Hout, pml, kH, i, j, k);
 }
 
-__global__ void __launch_bounds__(256) k_update_e(Grid g, const float *__restrict__ Ein,
+__global__ void __launch_bounds__(256, 8) k_update_e(Grid g, const float *__restrict__ Ein,
                                                   const float *__restrict__ Hnew,
                                                   float *__restrict__ Eout, Cpml pml, float kE,
-                                                  Source src, long long n) {
+                                                  Source src, const __grid_constant__ SourceStep ss) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     int j = blockIdx.y * blockDim.y + threadIdx.y;
     int k = blockIdx.z;
     if (i >= g.nx || j >= g.ny) return;
-    cell_e(g, Ein, Hnew, Eout, pml, kE, src, n, i, j, k);
+    cell_e(g, Ein, Hnew, Eout, pml, kE, src, ss, i, j, k);
 }
 
 void launch_update_h(const fdtd_ctx *h, cudaStream_t s) {
@@ -55,7 +55,8 @@ void launch_update_e(const fdtd_ctx *h, cudaStream_t s) {
     dim3 blk(32, 8, 1), grd((g.nx + 31) / 32, (g.ny + 7) / 8, g.nz);
     const float *in = h->fields[h->cur];
     float *out = h->fields[h->cur ^ 1];
-    k_update_e<<<grd, blk, 0, s>>>(g, in, out + 3 * g.comp, out, cpml_view(h), (float)h->kE, h->src, h->steps);
+    k_update_e<<<grd, blk, 0, s>>>(g, in, out + 3 * g.comp, out, cpml_view(h), (float)h->kE, h->src,
+                                   source_step(h->src, h->h_q.data(), h->steps));
 }
 
 __global__ void k_mur(Grid g, const float *__restrict__ Eold, float *__restrict__ Enew, float m) {

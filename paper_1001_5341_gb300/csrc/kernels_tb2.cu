@@ -1189,8 +1189,8 @@ void launch_tb2(fdtd_ctx *h, cudaStream_t s) {
     a.cur = h->cur;
     a.ecur = h->ecur;
     a.src = h->src;
-    a.ss1 = source_window(h->src, h->steps);
-    a.ss2 = source_window(h->src, h->steps + 1);
+    a.ss1 = source_step(h->src, h->h_q.data(), h->steps);
+    a.ss2 = source_step(h->src, h->h_q.data(), h->steps + 1);
     a.kE = (float)h->kE;
     a.kH = (float)h->kH;
     a.flags = h->d_flags;

@@ -154,7 +154,7 @@ void launch_vtile(fdtd_ctx *h, cudaStream_t s) {
     a.cur = h->cur;
     a.ecur = h->ecur;
     a.src = h->src;
-    a.ss = source_window(h->src, h->steps);
+    a.ss = source_step(h->src, h->h_q.data(), h->steps);
     a.kE = (float)h->kE;
     a.kH = (float)h->kH;
     a.flags = h->d_flags;

@@ -189,6 +189,13 @@ struct Blk {
     int nxb, xb;         // x boxes per array, floats per x box (128-byte aligned)
 };
 
+// whether the shower's footprint meets the tile (tile_block's numbering)
+__device__ __forceinline__ bool src_tile(const Args &A, int tile) {
+    const int i0 = tile % A.tiles_x * TXC, jb = tile / A.tiles_x * BY;
+    return A.src.active && i0 <= A.src.ic + A.src.L && i0 + TXC - 1 >= A.src.ic - A.src.L &&
+           jb <= A.src.jc + A.src.L && jb + BY - 1 >= A.src.jc - A.src.L;
+}
+
 __device__ __forceinline__ void issue_plane(const Args &A, const Maps &M, const Blk &B, float *st, uint64_t *bar,
                                             int r) {
     const int z = B.kstart + r;
@@ -659,8 +666,7 @@ __device__ __forceinline__ int tile_block(const Args &A, const Maps &M, int tile
     }
     B.kstart = B.k0 > 0 ? B.k0 - 1 : 0;
     B.nplanes = B.k1 - B.kstart + 1;   // input planes kstart .. k1
-    B.src_blk = A.src.active && B.i0 <= A.src.ic + A.src.L && B.i0 + TXC - 1 >= A.src.ic - A.src.L &&
-                B.jb <= A.src.jc + A.src.L && B.jb + BY - 1 >= A.src.jc - A.src.L;
+    B.src_blk = src_tile(A, tile);
     // which psi boxes the stages carry
     B.hx = B.hy = B.hz = false;
     B.l0 = 0;
