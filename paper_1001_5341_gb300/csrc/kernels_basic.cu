@@ -181,33 +181,61 @@ __device__ __forceinline__ bool kept(const Grid &g, int c, int i, int j, int k, 
     }
 }
 
-__global__ void k_set_field(Grid g, int c, const float *__restrict__ in, float *__restrict__ f,
-                            bool mur) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    int j = blockIdx.y, k = blockIdx.z;
-    if (i > g.nx) return;
-    long long s = ((long long)k * (g.ny + 1) + j) * (g.nx + 1) + i;
-    f[c * g.comp + gidx(g, i, j, k)] = kept(g, c, i, j, k, mur) ? in[s] : 0.0f;
+// Copies between a padded component and the caller's compact array, a warp per
+// COPY_ROWS consecutive x rows with its loads in flight together (the compact
+// rows of nx+1 floats are unaligned, so the accesses are 4-byte, coalesced).
+// Bound by HBM; one 128-thread block per row, as first written, was bound by
+// block launches: 69 us for 129 x 129 x 513, now 14.5 us (4.7 TB/s).
+constexpr int COPY_ROWS = 4, COPY_WARPS = 8;
+
+__global__ void __launch_bounds__(32 * COPY_WARPS) k_set_field(Grid g, int c, const float *__restrict__ in,
+                                                               float *__restrict__ f, bool mur) {
+    const long long rows = (long long)(g.ny + 1) * (g.nz + 1);
+    const long long r0 = ((long long)blockIdx.x * COPY_WARPS + (threadIdx.x >> 5)) * COPY_ROWS;
+    for (int i = threadIdx.x & 31; i <= g.nx; i += 32) {
+        float v[COPY_ROWS];
+#pragma unroll
+        for (int t = 0; t < COPY_ROWS; ++t)
+            if (r0 + t < rows) v[t] = in[(r0 + t) * (g.nx + 1) + i];
+#pragma unroll
+        for (int t = 0; t < COPY_ROWS; ++t)
+            if (r0 + t < rows) {
+                const int j = (int)((r0 + t) % (g.ny + 1)), k = (int)((r0 + t) / (g.ny + 1));
+                f[c * g.comp + gidx(g, i, j, k)] = kept(g, c, i, j, k, mur) ? v[t] : 0.0f;
+            }
+    }
 }
 
-__global__ void k_get_field(Grid g, int c, const float *__restrict__ f, float *__restrict__ out) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    int j = blockIdx.y, k = blockIdx.z;
-    if (i > g.nx) return;
-    long long s = ((long long)k * (g.ny + 1) + j) * (g.nx + 1) + i;
-    out[s] = f[c * g.comp + gidx(g, i, j, k)];
+__global__ void __launch_bounds__(32 * COPY_WARPS) k_get_field(Grid g, int c, const float *__restrict__ f,
+                                                               float *__restrict__ out) {
+    const long long rows = (long long)(g.ny + 1) * (g.nz + 1);
+    const long long r0 = ((long long)blockIdx.x * COPY_WARPS + (threadIdx.x >> 5)) * COPY_ROWS;
+    const float *s = f + c * g.comp + r0 * g.pitch;   // rows of a component are pitch floats apart
+    float *o = out + r0 * (g.nx + 1);
+    const int n = (int)(rows - r0 < COPY_ROWS ? rows - r0 : COPY_ROWS);
+    for (int i = threadIdx.x & 31; i <= g.nx; i += 32) {
+        float v[COPY_ROWS];
+#pragma unroll
+        for (int t = 0; t < COPY_ROWS; ++t)
+            if (t < n) v[t] = s[(long long)t * g.pitch + i];
+#pragma unroll
+        for (int t = 0; t < COPY_ROWS; ++t)
+            if (t < n) o[(long long)t * (g.nx + 1) + i] = v[t];
+    }
+}
+
+unsigned copy_blocks(const Grid &g) {
+    const long long rows = (long long)(g.ny + 1) * (g.nz + 1), per = COPY_ROWS * COPY_WARPS;
+    return (unsigned)((rows + per - 1) / per);
 }
 
 void launch_set_field(const fdtd_ctx *h, int comp, const float *compact, cudaStream_t s) {
-    const Grid &g = h->g;
-    dim3 blk(128), grd((g.nx + 1 + 127) / 128, g.ny + 1, g.nz + 1);
-    k_set_field<<<grd, blk, 0, s>>>(g, comp, compact, h->fields[h->cur], h->boundary == FDTD_MUR1);
+    k_set_field<<<copy_blocks(h->g), 32 * COPY_WARPS, 0, s>>>(h->g, comp, compact, h->fields[h->cur],
+                                                              h->boundary == FDTD_MUR1);
 }
 
 void launch_get_field(const fdtd_ctx *h, int comp, float *compact, cudaStream_t s) {
-    const Grid &g = h->g;
-    dim3 blk(128), grd((g.nx + 1 + 127) / 128, g.ny + 1, g.nz + 1);
-    k_get_field<<<grd, blk, 0, s>>>(g, comp, h->fields[h->cur], compact);
+    k_get_field<<<copy_blocks(h->g), 32 * COPY_WARPS, 0, s>>>(h->g, comp, h->fields[h->cur], compact);
 }
 
 // ---- energy / stability -----------------------------------------------------
