@@ -18,7 +18,8 @@
  *
  * The phase 2 pi f t_n is carried in 64-bit fixed point (the fraction of a
  * cycle), so it stays exact over any trace length; the sums run in float32
- * within a thread and in float64 across threads.  Status codes as in fdtd.h.
+ * over eight samples, in pairs of float32 within a thread and in float64 across
+ * threads.  Status codes as in fdtd.h.
  */
 #ifndef SPECTRA_GB300_H
 #define SPECTRA_GB300_H

@@ -121,3 +121,30 @@ def test_arguments(fd):
         assert call(*args) == -1, args
     with pytest.raises(ValueError):
         fd.trace_spectrum(torch.zeros(3, 4), 1e-11, f)
+
+
+@pytest.mark.parametrize("n_tr,n_t,n_f", [(1, 1, 1), (4, 7, 9), (5, 129, 130), (8, 640, 33), (9, 5003, 129), (17, 257, 8),
+                                          (3, 40001, 2), (33, 4096, 600), (200, 300, 1500)])
+def test_trace_and_frequency_groups(fd, n_tr, n_t, n_f):
+    """Sizes at the edges of the kernel's groups (traces, frequencies, tiles of
+    samples, clusters) and parameter tables carried by the launch or not."""
+    import torch
+    rng = np.random.default_rng(n_tr * n_t + n_f)
+    X = rng.standard_normal((n_tr, n_t, 2)).astype(np.float32)
+    coef = rng.standard_normal((n_tr, 2))
+    first = rng.integers(0, n_t, n_tr)
+    gate = np.stack([first, [rng.integers(0, n_t - f + 1) for f in first]], 1)
+    gate[-1] = 0, n_t
+    freqs = rng.uniform(-2e9, 2e9, n_f)
+    E = fd.trace_spectrum(torch.from_numpy(X).cuda(), 1.1e-11, freqs, t0=7e-11, coef=coef, gate=gate, taper=0.3)
+    _check(E.cpu().numpy().astype(np.complex128), X, 1.1e-11, freqs, 7e-11, coef, gate, 0.3)
+
+
+def test_non_finite_samples_stay_in_their_trace(fd):
+    import torch
+    X = np.ones((6, 300), dtype=np.float32)
+    X[1, 40], X[3, 50] = np.inf, np.nan
+    E = fd.trace_spectrum(torch.from_numpy(X).cuda(), 1e-11, [0.0, 3e8], gate=np.array([[0, 300]] * 5 + [[60, 100]])).cpu()
+    fin = torch.isfinite(torch.view_as_real(E)).all(-1)
+    assert fin[[0, 2, 4, 5]].all() and not fin[1].any() and not fin[3].any()
+    assert torch.isinf(E[1, 0].real)   # one infinite sample at frequency zero: an infinite sum
