@@ -73,9 +73,10 @@ int cyl_rings_gaussian(int n_rings, double d, double sigma_r, double *w);
 int cyl_set_probes(cyl_t h, const double *rz, int n, int max_steps);
 
 /*
- * Advance n >= 0 steps asynchronously on the handle's stream.  The
- * wavefront kernels advance K steps per launch; the n mod K steps left over
- * run on the two-kernel path.  FDTD_ERR_CAPACITY if detectors are set and
+ * Advance n >= 0 steps asynchronously on the handle's stream.  By default the
+ * steps run on tiles held in registers, up to K (8, 12 or 16) per launch.  With
+ * a wavefront kernel selected (cyl_set_kernel) K steps run per launch and the
+ * n mod K steps left over on the two-kernel path.  FDTD_ERR_CAPACITY if detectors are set and
  * the trace would overflow.
  */
 int cyl_step(cyl_t h, int n);
@@ -87,14 +88,16 @@ int cyl_step(cyl_t h, int n);
  * per lane, 2 = K 8 with 2, 3 = K 4 with 4, 4 = K 4 with 4 and registers
  * bounded for 4 blocks per SM, 5 = K 8 with 2 bounded the same way.
  * seg_rows = radial rows per warp segment (at most 1024), 0 picks it from the
- * grid and the SM count.  FDTD_ERR_ARG for another index.  The default
- * depends on the grid: 0 below 400000 cells (its steps are replayed from
- * captured graphs of 32 steps), 1 below 1600000 cells, 3 above.
+ * grid and the SM count.  FDTD_ERR_ARG for another index.  (Kernel 0 replays
+ * its steps from captured graphs of 32 steps.)  Until a kernel is selected the
+ * steps run on the tile path and cyl_kernel_info reports 0 below 400000 cells,
+ * 1 below 1600000 cells, 3 above.
  */
 int cyl_set_kernel(cyl_t h, int which, int seg_rows);
 
 /*
- * Autotuner of the wavefront kernel in use: it advances the simulation with
+ * Autotuner of the kernel in use.  On the tile path it times every tile size
+ * and K.  With a wavefront kernel it advances the simulation with
  * each candidate segment length (12 rows and up, in steps of 4 to 64, 8 to
  * 128 and 16 beyond, until the tiles fit one wave of the resident blocks; at
  * most 48 candidates), `launches` (1..8) launches each, times every launch
@@ -103,13 +106,16 @@ int cyl_set_kernel(cyl_t h, int which, int seg_rows);
  * detectors; the segment length decides how the work is cut, never what is
  * computed, so the fields and traces are those of any other length.  Returns
  * the steps it used in *steps_used (may be null): at most 48 x launches x K.
- * Nothing to do (0 steps) on the two-kernel path.  FDTD_ERR_CAPACITY, before
+ * Nothing to do (0 steps) where cyl_kernel_info reports kernel 0.  FDTD_ERR_CAPACITY, before
  * any step, if detectors are set and their trace has no room for those
  * steps; FDTD_ERR_ARG for launches outside 1..8.
  */
 int cyl_tune(cyl_t h, int launches, int *steps_used);
 
-/* The kernel in use, its steps per launch and rows per segment (any pointer may be null). */
+/*
+ * The kernel in use, its steps per launch and rows per segment (on the tile
+ * path: rows a tile owns); any pointer may be null.
+ */
 int cyl_kernel_info(cyl_t h, int *which, int *steps_per_launch, int *seg_rows);
 
 /* Name of the kernel in use (static string; "none" for a null handle). */

@@ -9,11 +9,14 @@
 // Cells outside a component's shape (E_r and H_phi on row nr, E_z and H_phi
 // on column nz) are never written either.
 //
-// Two paths advance the fields:
+// Three paths advance the fields:
+//  * the tile path (default): one launch advances up to K steps of tiles held in
+//    registers, reading the current set once and writing the other set once
+//    (24 bytes of DRAM per cell per launch; below, "Tile path");
 //  * the two-kernel path (one H launch and one E launch per step, in place on
 //    the current set; 36 bytes of DRAM per cell-update), which also runs the
-//    steps that are left when a step count is not a multiple of K;
-//  * the wavefront path (default): one launch advances K steps, reading the
+//    steps that the wavefront kernels leave when a count is not a multiple of K;
+//  * the wavefront path (cyl_set_kernel 1..5): one launch advances K steps, reading the
 //    current set once and writing the other set once (24 bytes per cell per
 //    launch).  Each warp owns a band of z columns and marches up the rows of
 //    one radial segment; time level s is computed one row behind level s-1,
@@ -33,12 +36,18 @@
 #include <cstring>
 #include <new>
 #include <numeric>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/cyl.h"
 #include "../../include/fdtd.h"
+#include "f32x2.cuh"
+#include "tma_pipe.cuh"
 
 namespace {
+
+using namespace fdtd::px2;
+using namespace fdtd::tma;
 
 constexpr double kC = 299792458.0;
 constexpr double kMu0 = 1.25663706212e-6;
@@ -60,17 +69,17 @@ struct Src {
     const float *coef;    // per ring: w_i / (eps A_i) (device)
 };
 
-__device__ __forceinline__ double src_q(const Src &s, double z) {
+__host__ __device__ __forceinline__ double src_q(const Src &s, const double *q, double z) {
     const double x = (z - s.z0) / s.bin_dz;
     if (!(x >= 0.0) || x > (double)(s.nbins - 1)) return 0.0;
     int b = (int)floor(x);
     if (b > s.nbins - 2) b = s.nbins - 2;
     const double f = x - (double)b;
-    return (1.0 - f) * s.q[b] + f * s.q[b + 1];
+    return (1.0 - f) * q[b] + f * q[b + 1];
 }
 
 // cumulative cloud-in-cell weight of the nodes <= j of a unit charge at z
-__device__ __forceinline__ double cum(double z, double d, int j) {
+__host__ __device__ __forceinline__ double cum(double z, double d, int j) {
     const double x = z / d;
     const double jj = floor(x);
     const double f = x - jj;
@@ -82,15 +91,15 @@ __device__ __forceinline__ double cum(double z, double d, int j) {
 
 // First face of the window of step n (n -> n+1); the deposit is zero outside
 // jlo .. jlo + MSRC - 1.
-__device__ __forceinline__ int src_jlo(const Src &s, long long n) {
+__host__ __device__ __forceinline__ int src_jlo(const Src &s, long long n) {
     const double za = s.z0 + s.v * (double)n * s.dt, zb = s.z0 + s.v * (double)(n + 1) * s.dt;
     return (int)floor(fmin(za, zb) / s.d) - 1;
 }
 
 // qbar dC_j of step n at face j+1/2, to be scaled by coef[i] for ring i.
-__device__ __forceinline__ float src_face(const Src &s, long long n, int j) {
+__host__ __device__ __forceinline__ float src_face(const Src &s, const double *q, long long n, int j) {
     const double za = s.z0 + s.v * (double)n * s.dt, zb = s.z0 + s.v * (double)(n + 1) * s.dt;
-    const double qb = src_q(s, s.z0 + s.v * ((double)n + 0.5) * s.dt);
+    const double qb = src_q(s, q, s.z0 + s.v * ((double)n + 0.5) * s.dt);
     return (float)(qb * (cum(zb, s.d, j) - cum(za, s.d, j)));
 }
 
@@ -144,7 +153,7 @@ __global__ void k_cyl_e(Dev D, float kE, float mur, int mur_on, Src S, const lon
         const float2 c = D.rowc[i];
         float ez1 = ez0 + c.x * Hp[o] - (i > 0 ? c.y * Hp[o - D.pitch] : 0.f);
         if (S.active && i < S.nw && (unsigned)(j - src_jlo(S, n)) < (unsigned)MSRC)
-            ez1 += S.coef[i] * src_face(S, n, j);
+            ez1 += S.coef[i] * src_face(S, S.q, n, j);
         Ez[o] = ez1;
         if (i == nr - 1) Ez[o + D.pitch] = mur_on ? ez0 + mur * (ez1 - Ez[o + D.pitch]) : 0.f;
     }
@@ -190,32 +199,6 @@ struct Wave {
     int nseg;                // segments; the last one runs to the wall
 };
 
-__device__ __forceinline__ uint32_t sa(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(sa(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(sa(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(sa(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// bounded: gives up after about two seconds of clock cycles
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const long long t0 = clock64();
-    while (!mbar_try_wait(bar, parity))
-        if (clock64() - t0 > (4LL << 30)) return false;
-    return true;
-}
 __device__ __forceinline__ void bulk_load(float *dst, const float *src, uint32_t bytes, uint64_t *bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                      sa(dst)),
@@ -467,7 +450,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_cyl_wave(Wave A) {
         const int s = tid / MSRC, m = tid % MSRC;
         const int jlo = src_jlo(A.src, A.n0 + s);
         if (m == 0) sjlo[s] = jlo;
-        ssrc[s][m] = src_face(A.src, A.n0 + s, jlo + m);
+        ssrc[s][m] = src_face(A.src, A.src.q, A.n0 + s, jlo + m);
     }
     if (lane == 0) {
         for (int s = 0; s < STAGES; ++s) mbar_init(&bars[wi][s], 1);
@@ -616,6 +599,421 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_cyl_wave(Wave A) {
     }
 }
 
+// ---------------------------------------------------------------------------
+// Tile path: K steps of a tile in registers
+// ---------------------------------------------------------------------------
+// A block of NWP warps holds a tile of 32 CPL columns by NWP R rows of the
+// three components in registers (lane L the columns CPL L .., warp w the rows
+// w R ..), advances it ks <= K steps and stores the cells that are K or more
+// from the tile's inner edges, which depend only on cells the tile held; the
+// tiles overlap by 2 K.  Where a tile ends at the axis, the wall or an end cap
+// there is no halo: its edge is the grid's.  Blocks take the tiles in turn,
+// one tensor copy (TMA) per tile, issued while the tile before it is stepped.
+//
+// Within a step every cell of a warp is in its own registers or a neighbour
+// lane's (shuffles); only the rows at the seam of two warps pass through
+// shared memory: E_z of a warp's first row to the warp below it, H_phi of its
+// last row to the warp above, each signalled on an mbarrier of its own.  Both
+// are computed first in their phase, so that a neighbour waits for them only
+// while the rest of the phase runs.  The order of waits keeps every barrier
+// within one phase of its waiter: a warp signals its last row of step s+1
+// after it has seen the first row of the warp above of step s, and that warp
+// writes it only once it has read the last row of step s; so one buffer per
+// seam suffices.
+//
+// The arithmetic runs on packed pairs (f32x2.cuh): 16 operations per four cells
+// and step.  Bound by instruction latency (three warps a scheduler at 160
+// registers: 41 % issue active) ahead of FP32 and, on grids beyond L2, DRAM
+// (24 bytes a cell and K steps).  Against the wavefront kernel and, below
+// 630^2 cells, the two kernels a step, us a step: 512^2 8.4 -> 1.32, 1024^2 8.0
+// -> 1.96, 2048^2 12.1 -> 5.6, 4096^2 28.3 -> 18.1, 8192^2 79 -> 64.  Also
+// timed: 6 or 4 rows a warp with 16 or 24 warps (within 5 % and 20 % slower),
+// 8 warps of 4 columns (spills), unpacked arithmetic (512^2 to 8192^2 6 to 17 %
+// slower), no early launch of the next kernel (8 % slower on one wave).
+constexpr int TK_MAX = 16;            // most steps per launch
+
+struct TileArgs {
+    int nr, nz, pitch;
+    Set out;
+    const float *ez_in;      // E_z of the input set (the wall row)
+    const float2 *rowc;
+    float kE, kH, mur;
+    int mur_on;
+    int K, ks;               // halo, steps of this launch
+    int ntx, ntiles;         // tile columns, tiles
+    int zset;                // first component of the input set in the tensor map
+    int nw;                  // source rows (0: none)
+    const float *coef;
+    int jlo[TK_MAX];         // first face of each step's deposit
+    float amp[TK_MAX][MSRC];
+    long long n0;
+    const int *poff;         // per tile and warp: first detector record
+    const int4 *prec;        // detector records (row in the warp, column in the tile, id, on the axis)
+    float *trace;
+    int max_steps;
+    int *flags;
+};
+
+template <int CPL, int NWP, int R>
+struct TGeo {
+    static constexpr int TC = 32 * CPL, TR = NWP * R, BOX = TC * TR;
+    static constexpr int XROW = NWP * TC;             // one exchange array: a row per warp
+    static constexpr size_t SMEM = sizeof(float) * (3 * BOX + 3 * XROW + 4 * TR) + 128;
+};
+
+// Start of tile t along an axis (tiles of T cells, halo K).
+__host__ __device__ inline int tile_at(int t, int T, int K) { return t * (T - 2 * K); }
+// Tiles along an axis of n cells.
+inline int tile_count(int n, int T, int K) { return n <= T ? 1 : (n - 2 * K + T - 2 * K - 1) / (T - 2 * K); }
+
+// The CPL columns of a lane as N = CPL / 2 pairs: pair n holds columns n and
+// n + N, so that a shift by one column is a renaming of pairs but for one of
+// them (one shuffle and one move).
+template <int N>
+__device__ __forceinline__ void from_cols(f32x2 (&p)[N], const float (&v)[2 * N]) {
+#pragma unroll
+    for (int n = 0; n < N; ++n) p[n] = pack(v[n], v[n + N]);
+}
+template <int N>
+__device__ __forceinline__ void to_cols(float (&v)[2 * N], const f32x2 (&p)[N]) {
+#pragma unroll
+    for (int n = 0; n < N; ++n) {
+        const float2 a = unpack(p[n]);
+        v[n] = a.x;
+        v[n + N] = a.y;
+    }
+}
+template <int N>
+__device__ __forceinline__ void load_cols(f32x2 (&p)[N], const float *s) {
+    if constexpr (N == 1) {
+        const float2 a = *reinterpret_cast<const float2 *>(s);
+        p[0] = pack(a.x, a.y);
+    } else {
+        static_assert(N == 2, "2 or 4 columns per lane");
+        const float4 a = *reinterpret_cast<const float4 *>(s);
+        p[0] = pack(a.x, a.z);
+        p[1] = pack(a.y, a.w);
+    }
+}
+// column j+1 (j-1) in the place of column j
+template <int N>
+__device__ __forceinline__ void shift_down(f32x2 (&o)[N], const f32x2 (&p)[N]) {
+    const float2 a = unpack(p[0]);
+    const float next = __shfl_down_sync(0xffffffffu, a.x, 1);
+#pragma unroll
+    for (int n = 0; n < N - 1; ++n) o[n] = p[n + 1];
+    o[N - 1] = pack(a.y, next);
+}
+template <int N>
+__device__ __forceinline__ void shift_up(f32x2 (&o)[N], const f32x2 (&p)[N]) {
+    const float2 a = unpack(p[N - 1]);
+    const float prev = __shfl_up_sync(0xffffffffu, a.y, 1);
+    o[0] = pack(prev, a.x);
+#pragma unroll
+    for (int n = 1; n < N; ++n) o[n] = p[n - 1];
+}
+
+template <int CPL, int NWP, int R, int MINB>
+__global__ void __launch_bounds__(32 * NWP, MINB)
+k_cyl_tile(const __grid_constant__ TileArgs A, const __grid_constant__ CUtensorMap M) {
+    typedef TGeo<CPL, NWP, R> G;
+    constexpr int TC = G::TC, TR = G::TR, NT = 32 * NWP;
+    constexpr unsigned ALL = 0xffffffffu;
+    extern __shared__ __align__(128) float smem[];
+    float *stage = smem;                       // [3][TR][TC]: E_r, E_z, H_phi of the next tile
+    float *xez = smem + 3 * G::BOX;            // E_z of each warp's first row
+    float *xh = xez + G::XROW;                 // H_phi of its last row
+    float *xer = xh + G::XROW;                 // E_r of its last row (detectors)
+    ulonglong2 *src = reinterpret_cast<ulonglong2 *>(xer + G::XROW);   // row coefficients of the tile, as pairs
+    constexpr int N = CPL / 2;                 // pairs per lane and row
+    const f32x2 nkE = pack(-A.kE, -A.kE), nkH = pack(-A.kH, -A.kH);
+    __shared__ __align__(8) uint64_t full, bez[NWP], bh[NWP];
+
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int nr = A.nr, nz = A.nz, K = A.K;
+    if (tid == 0) {
+        mbar_init(&full, 1);
+        for (int i = 0; i < NWP; ++i) {
+            mbar_init(&bez[i], 1);
+            mbar_init(&bh[i], 1);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    __syncthreads();
+    // the next launch may be set up while this one runs; this one has been, and
+    // waits here for the launch before it
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    auto fetch = [&](int tile) {
+        const int tx = tile % A.ntx, ty = tile / A.ntx;
+        mbar_expect_tx(&full, 3 * G::BOX * 4);
+        fdtd::tma::tma_load(stage, &M, &full, tile_at(tx, TC, K), tile_at(ty, TR, K), A.zset);
+    };
+    if (tid == 0 && (int)blockIdx.x < A.ntiles) fetch(blockIdx.x);
+
+    uint32_t ph = 0, pe = 0, pl = 0;   // parities: stage, E_z seam above, H seam below
+    bool ok = true, pending = (int)blockIdx.x < A.ntiles;   // pending: a copy is in flight
+    for (int tile = blockIdx.x; tile < A.ntiles; tile += gridDim.x) {
+        const int tx = tile % A.ntx, ty = tile / A.ntx;
+        const int c0 = tile_at(tx, TC, K), r0 = tile_at(ty, TR, K);
+        const bool last_x = tx == A.ntx - 1, last_y = tile + A.ntx >= A.ntiles;
+        const int col = c0 + lane * CPL, row = r0 + w * R;   // first column and row of the thread's cells
+        for (int t = tid; t < TR; t += NT) {
+            const float2 c = r0 + t < nr ? A.rowc[r0 + t] : make_float2(0.f, 0.f);
+            src[t] = make_ulonglong2(pack(c.x, c.x), pack(-c.y, -c.y));
+        }
+        f32x2 er[R][N], ez[R][N], h[R][N], wall[N];
+        if (ok) ok = mbar_wait(&full, ph);
+        if (ok) ph ^= 1u;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float *p = stage + (w * R + r) * TC + lane * CPL;
+            load_cols<N>(er[r], p);
+            load_cols<N>(ez[r], p + G::BOX);
+            load_cols<N>(h[r], p + 2 * G::BOX);
+        }
+        // the warp that holds row nr - 1 keeps the wall E_z(nr, j) too
+        const bool has_wall = last_y && row <= nr - 1 && nr - 1 < row + R;
+        const int rw = has_wall ? nr - 1 - row : -1;   // its row in the warp
+        if (has_wall) {
+            float v[CPL];
+#pragma unroll
+            for (int q = 0; q < CPL; ++q) v[q] = col + q < nz ? A.ez_in[(long long)nr * A.pitch + col + q] : 0.f;
+            from_cols<N>(wall, v);
+        }
+        if (!__syncthreads_and(ok)) break;     // the stage is read: its refill may start
+        const int next = tile + gridDim.x;
+        pending = next < A.ntiles;
+        if (tid == 0 && pending) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            fetch(next);
+        }
+        const bool caps = tx == 0 || last_x;   // the tile holds columns 0, 1 or nz - 1, nz
+        const bool rows = has_wall || row < A.nw;
+        int pbeg = 0, pend = 0;
+        if (A.poff) {
+            pbeg = A.poff[tile * NWP + w];
+            pend = A.poff[tile * NWP + w + 1];
+        }
+        const bool det = A.poff && A.poff[tile * NWP] < A.poff[tile * NWP + NWP];   // any in the tile
+
+        // detectors of step s (0-based) from the registers and E_r of the row below
+        auto detect = [&](int s) {
+            for (int pb = pbeg; pb < pend; pb += 32) {
+                const bool in = pb + lane < pend;
+                const int4 pr = in ? __ldg(&A.prec[pb + lane]) : make_int4(-1, 1, 0, 1);
+                const int l1 = pr.y / CPL, q1 = pr.y % CPL, l0 = (pr.y - 1) / CPL, q0 = (pr.y - 1) % CPL;
+                float ez1 = 0.f, ez0 = 0.f, er1 = 0.f, er0 = 0.f;
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    if (!__any_sync(ALL, pr.x == r)) continue;
+                    float vz[CPL], vr[CPL], vd[CPL];
+                    to_cols<N>(vz, ez[r]);
+                    to_cols<N>(vr, er[r]);
+                    to_cols<N>(vd, er[r > 0 ? r - 1 : 0]);
+#pragma unroll
+                    for (int q = 0; q < CPL; ++q) {
+                        const float a = __shfl_sync(ALL, vz[q], l1), b = __shfl_sync(ALL, vz[q], l0);
+                        const float c = __shfl_sync(ALL, vr[q], l1);
+                        const float d = r > 0 ? __shfl_sync(ALL, vd[q], l1) : 0.f;
+                        if (pr.x == r) {
+                            if (q == q1) { ez1 = a; er1 = c; er0 = d; }
+                            if (q == q0) ez0 = b;
+                        }
+                    }
+                }
+                if (in) {
+                    if (pr.x == 0 && w > 0) er0 = xer[(w - 1) * TC + pr.y / CPL * CPL + (q1 < N ? 2 * q1 : 2 * (q1 - N) + 1)];
+                    float *t = A.trace + ((long long)pr.z * A.max_steps + A.n0 + s) * 2;
+                    t[0] = 0.5f * (ez0 + ez1);
+                    t[1] = pr.w ? 0.f : 0.5f * (er0 + er1);
+                }
+            }
+        };
+        // a row of the warp's to an exchange array and back, in the order of its pairs
+        auto put = [&](float *x, const f32x2 (&v)[N]) {
+            f32x2 *p = reinterpret_cast<f32x2 *>(x + w * TC + lane * CPL);
+#pragma unroll
+            for (int n = 0; n < N; ++n) p[n] = v[n];
+        };
+        auto get = [&](const float *x, int row_w, f32x2 (&v)[N]) {
+            const f32x2 *p = reinterpret_cast<const f32x2 *>(x + row_w * TC + lane * CPL);
+#pragma unroll
+            for (int n = 0; n < N; ++n) v[n] = p[n];
+        };
+        auto sig = [&](uint64_t *b) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(b);
+        };
+        // H_phi(r, j) from E_r(r, j), E_r(r, j+1), E_z(r, j), E_z(r+1, j), the
+        // last row first; WALL: the warp holds row nr - 1
+        auto phase_h = [&](auto wall_c) {
+            constexpr bool WALL = decltype(wall_c)::value;
+#pragma unroll
+            for (int rr = 0; rr < R; ++rr) {
+                const int r = rr == 0 ? R - 1 : rr - 1;
+                f32x2 up[N], next[N];
+                if (r == R - 1) {
+                    // the top warp's last row lies in the halo, or past the wall
+                    get(xez, w < NWP - 1 ? w + 1 : w, up);
+                } else {
+#pragma unroll
+                    for (int n = 0; n < N; ++n) up[n] = ez[r < R - 1 ? r + 1 : r][n];
+                }
+                if (WALL && r == rw)
+#pragma unroll
+                    for (int n = 0; n < N; ++n) up[n] = wall[n];
+                shift_down<N>(next, er[r]);
+#pragma unroll
+                for (int n = 0; n < N; ++n)
+                    h[r][n] = fma2(nkH, sub2(sub2(next[n], er[r][n]), sub2(up[n], ez[r][n])), h[r][n]);
+                if (rr == 0 && w < NWP - 1) {
+                    put(xh, h[R - 1]);
+                    if (det) put(xer, er[R - 1]);   // of the step before
+                    sig(&bh[w]);
+                }
+            }
+        };
+        // E_z(r, j) from H_phi(r, j), H_phi(r-1, j) (on the axis cB = 0), E_r(r, j)
+        // from H_phi(r, j-1), H_phi(r, j).  CAPS: the tile holds columns 0, 1 or
+        // nz - 1, nz; ROWS: the warp holds source rows or row nr - 1.
+        auto phase_e = [&](auto caps_c, auto rows_c, int s) {
+            constexpr bool CAPS = decltype(caps_c)::value, ROWS = decltype(rows_c)::value;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const ulonglong2 c = src[w * R + r];   // (cA, cA), (-cB, -cB)
+                if (ROWS && r == rw)   // the old values first
+#pragma unroll
+                    for (int n = 0; n < N; ++n) wall[n] = A.mur_on ? fma2(pack(-A.mur, -A.mur), wall[n], ez[r][n]) : 0ull;
+                f32x2 lower[N];
+                if (r == 0) {
+                    get(xh, w > 0 ? w - 1 : 0, lower);   // the lowest warp's first row: cB = 0 on the axis, else halo
+                } else {
+#pragma unroll
+                    for (int n = 0; n < N; ++n) lower[n] = h[r > 0 ? r - 1 : 0][n];
+                }
+#pragma unroll
+                for (int n = 0; n < N; ++n) ez[r][n] = fma2(c.y, lower[n], fma2(c.x, h[r][n], ez[r][n]));
+                if (ROWS && row + r < A.nw) {
+                    const float cf = __ldg(&A.coef[row + r]);
+                    const int jlo = A.jlo[s];
+                    float v[CPL];
+                    to_cols<N>(v, ez[r]);
+#pragma unroll
+                    for (int q = 0; q < CPL; ++q) {
+                        const unsigned m = (unsigned)(col + q - jlo);
+                        if (m < (unsigned)MSRC) v[q] += cf * A.amp[s][m];
+                    }
+                    from_cols<N>(ez[r], v);
+                }
+                if (ROWS && r == rw && A.mur_on)
+#pragma unroll
+                    for (int n = 0; n < N; ++n) wall[n] = fma2(pack(A.mur, A.mur), ez[r][n], wall[n]);
+                if (r == 0 && w > 0) {
+                    put(xez, ez[0]);
+                    sig(&bez[w]);
+                }
+                f32x2 prev[N], old[N];
+                shift_up<N>(prev, h[r]);
+#pragma unroll
+                for (int n = 0; n < N; ++n) {
+                    old[n] = er[r][n];
+                    er[r][n] = fma2(nkE, sub2(h[r][n], prev[n]), er[r][n]);
+                }
+                if (CAPS) {   // from the columns next to the caps, old and new
+                    float o[CPL], v[CPL];
+                    to_cols<N>(o, old);
+                    to_cols<N>(v, er[r]);
+                    if (col == 0) v[0] = A.mur_on ? o[1] + A.mur * (v[1] - o[0]) : 0.f;
+                    const float old_l = __shfl_up_sync(ALL, o[CPL - 1], 1);
+                    const float new_l = __shfl_up_sync(ALL, v[CPL - 1], 1);
+#pragma unroll
+                    for (int q = 0; q < CPL; ++q)
+                        if (col + q == nz) {
+                            const float ol = q > 0 ? o[q > 0 ? q - 1 : 0] : old_l;
+                            const float nl = q > 0 ? v[q > 0 ? q - 1 : 0] : new_l;
+                            v[q] = A.mur_on ? ol + A.mur * (nl - o[q]) : 0.f;
+                        }
+                    from_cols<N>(er[r], v);
+                }
+            }
+        };
+        const std::true_type yes{};
+        const std::false_type no{};
+        put(xez, ez[0]);
+        if (w > 0) sig(&bez[w]);
+        __syncwarp();
+        for (int s = 0; s < A.ks; ++s) {
+            if (w < NWP - 1) {
+                if (ok) ok = mbar_wait(&bez[w + 1], pe);
+                pe ^= 1u;
+            }
+            if (has_wall) phase_h(yes);
+            else phase_h(no);
+            if (w > 0) {
+                if (ok) ok = mbar_wait(&bh[w - 1], pl);
+                pl ^= 1u;
+            }
+            if (det && s > 0) {
+                detect(s - 1);
+                __syncwarp();
+            }
+            if (rows) phase_e(yes, yes, s);
+            else if (caps) phase_e(yes, no, s);
+            else phase_e(no, no, s);
+        }
+        // the E_z seams were signalled once more than they were waited for, and
+        // the detectors of the last step need the E_r rows of the warps below
+        if (w < NWP - 1) {
+            if (ok) ok = mbar_wait(&bez[w + 1], pe);
+            pe ^= 1u;
+            if (det) {
+                put(xer, er[R - 1]);
+                sig(&bh[w]);
+            }
+        }
+        if (det) {
+            if (w > 0) {
+                if (ok) ok = mbar_wait(&bh[w - 1], pl);
+                pl ^= 1u;
+            }
+            detect(A.ks - 1);
+        }
+        // owned cells
+        const int oc0 = tx > 0 ? c0 + K : 0, oc1 = last_x ? nz + 1 : c0 + TC - K;
+        const int or0 = ty > 0 ? r0 + K : 0, or1 = last_y ? nr : r0 + TR - K;
+        if (col >= oc0 && col < oc1) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int i = row + r;
+                if (i < or0 || i >= or1) continue;
+                const long long o = (long long)i * A.pitch + col;
+                float v[CPL];
+                to_cols<N>(v, er[r]);
+                st_cols<CPL>(A.out.Er + o, v, nz + 1 - col);
+                to_cols<N>(v, h[r]);
+                st_cols<CPL>(A.out.Hp + o, v, nz - col);
+                to_cols<N>(v, ez[r]);
+                st_cols<CPL>(A.out.Ez + o, v, nz - col);
+                if (r == rw) {
+                    to_cols<N>(v, wall);
+                    st_cols<CPL>(A.out.Ez + o + A.pitch, v, nz - col);
+                }
+            }
+        }
+        __syncthreads();   // the exchange rows and coefficients are done with
+    }
+    if (__syncthreads_or(!ok) && tid == 0) {
+        // a wait expired: record it; a copy still in flight after these waits may
+        // land after the block ends: flag bit 8 (the handle's status is sticky)
+        atomicOr(A.flags, 1);
+        bool landed = !pending;
+        for (int t = 0; t < 4 && !landed; ++t) landed = mbar_wait(&full, ph);
+        if (!landed) atomicOr(A.flags, 8);
+    }
+}
+
 struct Variant {
     int K, CPL, stages;
     void (*fn)(Wave);
@@ -669,6 +1067,14 @@ struct cyl_ctx {
     cudaEvent_t gev;
     cudaGraphExec_t g2k[2];
     bool graph_off;
+    // tile path: on unless a kernel was selected (cyl_set_kernel)
+    bool tile;
+    int tv, tK, tslots;      // variant, halo (steps per launch), resident blocks
+    int ntx, nty;
+    CUtensorMap tmap;
+    int *d_tpoff;            // detector records (null: no detectors)
+    int4 *d_tprec;
+    std::vector<double> h_q; // the charge table, for each launch's deposit
     unsigned *d_tiles;       // wavefront tile counters (next tile, blocks done)
     int slots;               // resident blocks of the wavefront kernel in use
 };
@@ -692,11 +1098,19 @@ void free_src(cyl_ctx *h) {
     h->src = Src{};
 }
 
+void free_tile_probes(cyl_ctx *h) {
+    if (h->d_tpoff) cudaFree(h->d_tpoff);
+    if (h->d_tprec) cudaFree(h->d_tprec);
+    h->d_tpoff = nullptr;
+    h->d_tprec = nullptr;
+}
+
 void free_probes(cyl_ctx *h) {
     if (h->d_ij) cudaFree(h->d_ij);
     if (h->d_trace) cudaFree(h->d_trace);
     if (h->d_poff) cudaFree(h->d_poff);
     if (h->d_prec) cudaFree(h->d_prec);
+    free_tile_probes(h);
     h->d_ij = nullptr;
     h->d_trace = nullptr;
     h->d_poff = nullptr;
@@ -814,10 +1228,153 @@ int configure(cyl_ctx *h, int which, int seg_rows) {
     return build_wave_probes(h);
 }
 
-// Default kernel by grid size (measured on the Table I grids): below about
-// 630^2 cells the two-kernel path replayed from graphs (the wavefront's warps
-// are too few to hide their step latency), up to about 1250^2 the wavefront
-// with 2 columns per lane (twice the warps), above it 4 columns per lane.
+struct TVariant {
+    int TC, TR, NWP, R;
+    size_t smem;
+    void (*fn)(TileArgs, CUtensorMap);
+    const char *name;
+};
+template <int CPL, int NWP, int R, int MINB>
+TVariant tvariant(const char *name) {
+    typedef TGeo<CPL, NWP, R> G;
+    return TVariant{G::TC, G::TR, NWP, R, G::SMEM, k_cyl_tile<CPL, NWP, R, MINB>, name};
+}
+const TVariant kTiles[] = {tvariant<4, 12, 8, 1>("k_cyl_tile<4,12,8>"), tvariant<2, 16, 4, 1>("k_cyl_tile<2,16,4>")};
+constexpr int kNumTiles = 2;
+constexpr int kTileK[] = {8, 12, 16};   // halos (steps per launch); multiples of the columns per lane
+
+// Detector records of the tile path: per tile and warp, in the warp that holds
+// the detector's row.
+int build_tile_probes(cyl_ctx *h) {
+    free_tile_probes(h);
+    if (h->np == 0) return FDTD_OK;
+    const TVariant &v = kTiles[h->tv];
+    const int K = h->tK, ntiles = h->ntx * h->nty;
+    auto tile_of = [&](int i, int T, int n) { return std::min(std::max(i - K, 0) / (T - 2 * K), n - 1); };
+    std::vector<int> off((size_t)ntiles * v.NWP + 1, 0), key(h->np);
+    std::vector<int4> val(h->np), rec(h->np);
+    for (int p = 0; p < h->np; ++p) {
+        const int i = h->pij[2 * p], j = h->pij[2 * p + 1];
+        const int tx = tile_of(j, v.TC, h->ntx), ty = tile_of(i, v.TR, h->nty);
+        const int r = i - tile_at(ty, v.TR, K), c = j - tile_at(tx, v.TC, K);
+        key[p] = (ty * h->ntx + tx) * v.NWP + r / v.R;
+        val[p] = make_int4(r % v.R, c, p, i == 0);
+        off[key[p] + 1]++;
+    }
+    for (size_t k = 1; k < off.size(); ++k) off[k] += off[k - 1];
+    std::vector<int> at(off.begin(), off.end() - 1);
+    for (int p = 0; p < h->np; ++p) rec[at[key[p]]++] = val[p];
+    if (cudaMalloc(&h->d_tpoff, off.size() * sizeof(int)) != cudaSuccess ||
+        cudaMalloc(&h->d_tprec, rec.size() * sizeof(int4)) != cudaSuccess) {
+        cudaGetLastError();
+        return FDTD_ERR_OOM;
+    }
+    if (note(h, cudaMemcpy(h->d_tpoff, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice)) != FDTD_OK ||
+        note(h, cudaMemcpy(h->d_tprec, rec.data(), rec.size() * sizeof(int4), cudaMemcpyHostToDevice)) != FDTD_OK)
+        return FDTD_ERR_CUDA;
+    return FDTD_OK;
+}
+
+// Tiles, tensor map and detector records of tile variant tv with halo K.
+int configure_tile(cyl_ctx *h, int tv, int K) {
+    const TVariant &v = kTiles[tv];
+    h->tv = tv;
+    h->tK = K;
+    h->ntx = tile_count(h->nz + 1, v.TC, K);
+    h->nty = tile_count(h->nr, v.TR, K);
+    int dev = 0, sms = 152, per_sm = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, v.fn, 32 * v.NWP, v.smem) != cudaSuccess || per_sm < 1) {
+        cudaGetLastError();
+        return FDTD_ERR_CUDA;
+    }
+    h->tslots = sms * per_sm;
+    fdtd::tma::EncodeTiled encode = fdtd::tma::encoder();
+    const cuuint64_t dims[3] = {(cuuint64_t)h->nz + 1, (cuuint64_t)h->nr + 1, 6};
+    const cuuint64_t strides[2] = {(cuuint64_t)h->pitch * 4, (cuuint64_t)h->comp * 4};
+    const cuuint32_t box[3] = {(cuuint32_t)v.TC, (cuuint32_t)v.TR, 3}, one[3] = {1, 1, 1};
+    if (!encode || encode(&h->tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, h->block + PADL, dims, strides, box, one,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return FDTD_ERR_CUDA;
+    return build_tile_probes(h);
+}
+
+// Steps n .. n + ks - 1 (ks <= tK) on the tile path.
+void launch_tile(cyl_ctx *h, int ks) {
+    const TVariant &v = kTiles[h->tv];
+    TileArgs A{};
+    A.nr = h->nr;
+    A.nz = h->nz;
+    A.pitch = h->pitch;
+    A.out = h->set[h->cur ^ 1];
+    A.ez_in = h->set[h->cur].Ez;
+    A.rowc = h->d_rowc;
+    A.kE = (float)h->kE;
+    A.kH = (float)h->kH;
+    A.mur = (float)h->mur;
+    A.mur_on = h->boundary == FDTD_MUR1;
+    A.K = h->tK;
+    A.ks = ks;
+    A.ntx = h->ntx;
+    A.ntiles = h->ntx * h->nty;
+    A.zset = 3 * h->cur;
+    if (h->src.active) {
+        A.nw = h->src.nw;
+        A.coef = h->src.coef;
+        for (int s = 0; s < ks; ++s) {
+            A.jlo[s] = src_jlo(h->src, h->steps + s);
+            for (int m = 0; m < MSRC; ++m) A.amp[s][m] = src_face(h->src, h->h_q.data(), h->steps + s, A.jlo[s] + m);
+        }
+    }
+    A.n0 = h->steps;
+    A.poff = h->d_tpoff;
+    A.prec = h->d_tprec;
+    A.trace = h->d_trace;
+    A.max_steps = h->max_steps;
+    A.flags = h->d_flags;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(std::min(A.ntiles, std::max(1, h->tslots)));
+    cfg.blockDim = dim3(32 * v.NWP);
+    cfg.dynamicSmemBytes = v.smem;
+    cfg.stream = h->stream;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    note(h, cudaLaunchKernelEx(&cfg, v.fn, A, h->tmap));
+    h->launches++;
+    h->cur ^= 1;
+    h->steps += ks;
+    h->step_ok = false;
+}
+
+// Tile variant and halo by grid size: the least time per step of a model,
+// (waves of tiles x (a K + b) + c) / K us on 152 SMs, fitted to GB300 times of
+// square grids from 256 to 8192 a side: the larger tile (fewer halo cells)
+// (0.9 K + 2.9) a wave and 8, the smaller (0.7 K + 0.6) and 5.  It picks the
+// measured best on 512 (the smaller, K 8: 1.32 us a step against 1.80), 1024
+// (K 12: 1.96 against 2.18), 2048 (K 12: 5.6 against 7.3) and 4096, 8192 (K 8:
+// 18.1 and 64.0, K 12 19.0 and 67.8); cyl_tune times them all.
+void tile_default(int nr, int nz, int &tv, int &K) {
+    static const double cost[kNumTiles][3] = {{0.9, 2.9, 8.0}, {0.7, 0.6, 5.0}};
+    double best = 1e300;
+    for (int v = 0; v < kNumTiles; ++v)
+        for (int k : kTileK) {
+            const double tiles = (double)tile_count(nz + 1, kTiles[v].TC, k) * tile_count(nr, kTiles[v].TR, k);
+            const double t = (std::ceil(tiles / 152.0) * (cost[v][0] * k + cost[v][1]) + cost[v][2]) / k;
+            if (t < best) {
+                best = t;
+                tv = v;
+                K = k;
+            }
+        }
+}
+
+// The kernel index that a handle reports before cyl_set_kernel, by grid size;
+// its steps run on the tile path.
 int default_kernel(int nr, int nz) {
     const long long cells = (long long)nr * nz;
     return cells < 400000 ? 0 : cells < 1600000 ? 1 : 3;
@@ -1004,7 +1561,15 @@ int cyl_create(cyl_t *out, int nr, int nz, double d, double dt, double eps_r, in
     note(h, cudaMemsetAsync(h->d_flags, 0, sizeof(int), h->stream));
     note(h, cudaMemcpyAsync(h->d_rowc, rowc.data(), rowc.size() * sizeof(float2), cudaMemcpyHostToDevice, h->stream));
     note(h, cudaStreamSynchronize(h->stream));
+    for (const TVariant &v : kTiles)
+        note(h, cudaFuncSetAttribute(v.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v.smem));
     if (h->status == FDTD_OK) h->status = configure(h, default_kernel(nr, nz), 0);
+    if (h->status == FDTD_OK) {
+        int tv = 0, tK = 8;
+        tile_default(nr, nz, tv, tK);
+        h->status = configure_tile(h, tv, tK);
+        h->tile = h->status == FDTD_OK;
+    }
     if (h->status != FDTD_OK) {
         const int st = h->status;
         cyl_destroy(h);
@@ -1035,6 +1600,7 @@ int cyl_set_kernel(cyl_t h, int which, int seg_rows) {
     if (h->status != FDTD_OK) return h->status;
     const int st = configure(h, which, seg_rows);
     if (st != FDTD_OK && h->status == FDTD_OK) h->status = st;
+    h->tile = false;
     return st;
 }
 int cyl_tune(cyl_t h, int launches, int *steps_used) {
@@ -1042,20 +1608,30 @@ int cyl_tune(cyl_t h, int launches, int *steps_used) {
     if (!h || launches < 1 || launches > 8) return FDTD_ERR_ARG;
     if (h->status != FDTD_OK) return h->status;
     if (h->kernel == 0) return FDTD_OK;   // the two-kernel path has no segments
-    // candidates: 12 rows and up (steps of 4 to 64, 8 to 128, 16 beyond) until
-    // the tiles fit one wave of the resident blocks (longer segments then only
-    // lengthen every tile); at most TUNE_MAX of them
+    // candidates of the wavefront kernels: 12 rows and up (steps of 4 to 64, 8
+    // to 128, 16 beyond) until the tiles fit one wave of the resident blocks
+    // (longer segments then only lengthen every tile), at most TUNE_MAX of
+    // them; of the tile path: every variant and halo
     const long long bx = (h->nbands + NW - 1) / NW;
     const long long slots = std::max(1, h->slots);
     std::vector<int> cand;
-    for (int L = 12; L <= std::min(h->nr + 1, LMAX) && (int)cand.size() < TUNE_MAX;
-         L += L < 64 ? 4 : L < 128 ? 8 : 16) {
-        cand.push_back(L);
-        long long nseg = (h->nr + 1 + L - 1) / L;
-        if (nseg > 1 && (h->nr + 1) % L == 1) --nseg;
-        if (nseg * bx <= slots) break;
+    long long need = 0;
+    if (h->tile) {
+        for (int v = 0; v < kNumTiles; ++v)
+            for (int k : kTileK) {
+                cand.push_back(v * (TK_MAX + 1) + k);
+                need += (long long)launches * k;
+            }
+    } else {
+        for (int L = 12; L <= std::min(h->nr + 1, LMAX) && (int)cand.size() < TUNE_MAX;
+             L += L < 64 ? 4 : L < 128 ? 8 : 16) {
+            cand.push_back(L);
+            long long nseg = (h->nr + 1 + L - 1) / L;
+            if (nseg > 1 && (h->nr + 1) % L == 1) --nseg;
+            if (nseg * bx <= slots) break;
+        }
+        need = (long long)cand.size() * launches * h->K;
     }
-    const long long need = (long long)cand.size() * launches * h->K;
     if (h->np > 0 && h->steps + need > h->max_steps) return FDTD_ERR_CAPACITY;
     std::vector<cudaEvent_t> ev(launches + 1, nullptr);
     for (auto &e : ev)
@@ -1066,33 +1642,38 @@ int cyl_tune(cyl_t h, int launches, int *steps_used) {
             return FDTD_ERR_CUDA;
         }
     const int kernel = h->kernel;
-    int best = h->L;
-    float best_ms = -1.f;
+    auto select = [&](int c) {
+        return h->tile ? configure_tile(h, c / (TK_MAX + 1), c % (TK_MAX + 1)) : configure(h, kernel, c);
+    };
+    int best = h->tile ? h->tv * (TK_MAX + 1) + h->tK : h->L;
+    float best_ms = -1.f;   // per step
     int used = 0;
-    for (int L : cand) {
-        if (configure(h, kernel, L) != FDTD_OK) break;
+    for (int c : cand) {
+        if (select(c) != FDTD_OK) break;
+        const int K = h->tile ? h->tK : h->K;
         cudaEventRecord(ev[0], h->stream);
         for (int i = 0; i < launches; ++i) {
-            launch_wave(h);
+            if (h->tile) launch_tile(h, K);
+            else launch_wave(h);
             cudaEventRecord(ev[i + 1], h->stream);
         }
-        used += launches * h->K;
+        used += launches * K;
         if (note(h, cudaEventSynchronize(ev[launches])) != FDTD_OK || h->status != FDTD_OK) break;
         float ms = -1.f;   // the fastest launch of the candidate
         for (int i = 0; i < launches; ++i) {
             float t = 0.f;
             if (cudaEventElapsedTime(&t, ev[i], ev[i + 1]) == cudaSuccess && (ms < 0.f || t < ms)) ms = t;
         }
-        if (ms >= 0.f && (best_ms < 0.f || ms < best_ms)) {
-            best_ms = ms;
-            best = L;
+        if (ms >= 0.f && (best_ms < 0.f || ms / K < best_ms)) {
+            best_ms = ms / K;
+            best = c;
         }
     }
     for (auto &e : ev) cudaEventDestroy(e);
     cudaGetLastError();
     if (steps_used) *steps_used = used;
     if (h->status != FDTD_OK) return h->status;
-    const int st = configure(h, kernel, best);
+    const int st = select(best);
     if (st != FDTD_OK && h->status == FDTD_OK) h->status = st;
     return st;
 }
@@ -1100,8 +1681,8 @@ int cyl_tune(cyl_t h, int launches, int *steps_used) {
 int cyl_kernel_info(cyl_t h, int *which, int *steps_per_launch, int *seg_rows) {
     if (!h) return FDTD_ERR_ARG;
     if (which) *which = h->kernel;
-    if (steps_per_launch) *steps_per_launch = h->K;
-    if (seg_rows) *seg_rows = h->L;
+    if (steps_per_launch) *steps_per_launch = h->tile ? h->tK : h->K;
+    if (seg_rows) *seg_rows = h->tile ? kTiles[h->tv].TR - 2 * h->tK : h->L;
     return FDTD_OK;
 }
 
@@ -1128,6 +1709,12 @@ int cyl_set_shower(cyl_t h, const double *q, int n_bins, double z0, double bin_d
     if (note(h, cudaMemcpy(h->d_q, q, n_bins * sizeof(double), cudaMemcpyHostToDevice)) != FDTD_OK ||
         note(h, cudaMemcpy(h->d_coef, coef.data(), nw * sizeof(float), cudaMemcpyHostToDevice)) != FDTD_OK)
         return h->status;
+    try {
+        h->h_q.assign(q, q + n_bins);
+    } catch (const std::bad_alloc &) {
+        free_src(h);
+        return FDTD_ERR_OOM;
+    }
     h->src.active = 1;
     h->src.nbins = n_bins;
     h->src.nw = std::min(nw, h->nr);   // ring nr lies on the wall, whose E_z the boundary sets
@@ -1157,7 +1744,8 @@ int cyl_set_probes(cyl_t h, const double *rz, int n, int max_steps) {
     free_probes(h);
     if (n == 0) {
         // the wavefront kernel reads its (empty) per-warp lists
-        const int st = build_wave_probes(h);
+        int st = build_wave_probes(h);
+        if (st == FDTD_OK) st = build_tile_probes(h);
         if (st != FDTD_OK && h->status == FDTD_OK) h->status = st;
         return st;
     }
@@ -1173,7 +1761,8 @@ int cyl_set_probes(cyl_t h, const double *rz, int n, int max_steps) {
     h->pij = ij;
     h->np = n;
     h->max_steps = max_steps;
-    const int st = build_wave_probes(h);
+    int st = build_wave_probes(h);
+    if (st == FDTD_OK) st = build_tile_probes(h);
     if (st != FDTD_OK && h->status == FDTD_OK) h->status = st;
     return st;
 }
@@ -1182,6 +1771,7 @@ int cyl_step(cyl_t h, int n) {
     if (!h || n < 0) return FDTD_ERR_ARG;
     if (h->status != FDTD_OK) return h->status;
     if (h->np > 0 && h->steps + n > h->max_steps) return FDTD_ERR_CAPACITY;
+    for (; h->tile && n > 0; n -= std::min(n, h->tK)) launch_tile(h, std::min(n, h->tK));
     if (h->kernel > 0)
         for (; n >= h->K; n -= h->K) launch_wave(h);
     if (n > 0) launch_two_kernel(h, n);
@@ -1252,7 +1842,7 @@ int cyl_reset(cyl_t h) {
     return cyl_sync(h);
 }
 
-const char *cyl_kernel_name(cyl_t h) { return h ? kVariants[h->kernel].name : "none"; }
+const char *cyl_kernel_name(cyl_t h) { return !h ? "none" : h->tile ? kTiles[h->tv].name : kVariants[h->kernel].name; }
 
 int cyl_steps_done(cyl_t h, int64_t *steps) {
     if (!h || !steps) return FDTD_ERR_ARG;
