@@ -96,7 +96,10 @@ int vtile_prepare(fdtd_ctx *h) {
     // planes between them in m chunks of cm.  With one block per SM, the
     // middle blocks run in ceil(tiles m / SMs) waves of about cm + 4 plane
     // times each (warm-up plane and pipeline fill); m minimises that, chunks
-    // of at least 16 planes.  More chunks where the coefficient table of a
+    // of at least 16 planes on a CPML grid and 4 on others: with 16 a 96^3 Mur
+    // grid ran on 72 of 152 SMs (30.9 us a step, now 22.7; 60 x 200 x 64 Mur 32.9
+    // -> 28.8, 100^3 PEC 27.8 -> 20.6), but on a CPML grid the layer blocks then
+    // make a second wave (64 x 56 x 200: 40.1 -> 53.8).  More chunks where the coefficient table of a
     // long chunk leaves the ring too small for two of the largest stages.
     const int mid = P > 0 ? g.nz - 2 * P - 1 : g.nz;
     const long long sms = h->num_sms > 0 ? h->num_sms : 1;
@@ -105,7 +108,7 @@ int vtile_prepare(fdtd_ctx *h) {
     // through L2 only while they stay within a few planes of each other
     constexpr long long CM_MAX = 160;
     const long long m_lo = std::max(1LL, (mid + CM_MAX - 1) / CM_MAX);
-    const long long m_hi = std::max(m_lo, (long long)(mid / 16));
+    const long long m_hi = std::max(m_lo, (long long)(mid / (P > 0 ? 16 : 4)));
     long long m = m_lo, best = -1;
     for (long long mm = m_lo; mm <= m_hi; ++mm) {
         const long long cm = (mid + mm - 1) / mm;
