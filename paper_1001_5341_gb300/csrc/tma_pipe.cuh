@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "f32x2.cuh"
+
 namespace fdtd {
 namespace tma {
 
@@ -58,12 +60,19 @@ __device__ __forceinline__ void tma_load(float *dst, const CUtensorMap *map, uin
 __device__ __forceinline__ float4 lds4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
 __device__ __forceinline__ void sts4(float *p, float4 v) { *reinterpret_cast<float4 *>(p) = v; }
 
+// the field update on packed pairs (x, y) and (z, w)
+__device__ __forceinline__ float4 join(px2::f32x2 lo, px2::f32x2 hi) {
+    const float2 a = px2::unpack(lo), b = px2::unpack(hi);
+    return make_float4(a.x, a.y, b.x, b.y);
+}
 __device__ __forceinline__ float4 operator-(float4 a, float4 b) {
-    return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
+    return join(px2::sub2(px2::pack(a.x, a.y), px2::pack(b.x, b.y)), px2::sub2(px2::pack(a.z, a.w), px2::pack(b.z, b.w)));
 }
 // a + s * d, elementwise
 __device__ __forceinline__ float4 axpy(float4 a, float s, float4 d) {
-    return make_float4(a.x + s * d.x, a.y + s * d.y, a.z + s * d.z, a.w + s * d.w);
+    const px2::f32x2 ss = px2::pack(s, s);
+    return join(px2::fma2(ss, px2::pack(d.x, d.y), px2::pack(a.x, a.y)),
+                px2::fma2(ss, px2::pack(d.z, d.w), px2::pack(a.z, a.w)));
 }
 
 // CPML recursion psi <- b psi + a d; the derivative becomes d + psi
@@ -71,14 +80,20 @@ __device__ __forceinline__ float cpml1(float &psi, float a, float b, float d) {
     psi = b * psi + a * d;
     return d + psi;
 }
-__device__ __forceinline__ float4 cpml4(float4 &psi, float a, float b, float4 d) {
-    return make_float4(cpml1(psi.x, a, b, d.x), cpml1(psi.y, a, b, d.y), cpml1(psi.z, a, b, d.z),
-                       cpml1(psi.w, a, b, d.w));
+__device__ __forceinline__ px2::f32x2 cpml2(px2::f32x2 &psi, px2::f32x2 a, px2::f32x2 b, px2::f32x2 d) {
+    psi = px2::fma2(b, psi, px2::mul2(a, d));
+    return px2::add2(d, psi);
 }
 // elementwise coefficients
 __device__ __forceinline__ float4 cpmlv(float4 &psi, float4 a, float4 b, float4 d) {
-    return make_float4(cpml1(psi.x, a.x, b.x, d.x), cpml1(psi.y, a.y, b.y, d.y), cpml1(psi.z, a.z, b.z, d.z),
-                       cpml1(psi.w, a.w, b.w, d.w));
+    px2::f32x2 p = px2::pack(psi.x, psi.y), q = px2::pack(psi.z, psi.w);
+    const float4 r = join(cpml2(p, px2::pack(a.x, a.y), px2::pack(b.x, b.y), px2::pack(d.x, d.y)),
+                          cpml2(q, px2::pack(a.z, a.w), px2::pack(b.z, b.w), px2::pack(d.z, d.w)));
+    psi = join(p, q);
+    return r;
+}
+__device__ __forceinline__ float4 cpml4(float4 &psi, float a, float b, float4 d) {
+    return cpmlv(psi, make_float4(a, a, a, a), make_float4(b, b, b, b), d);
 }
 
 // zero the whole vector (all) or its first element (first): the components a
