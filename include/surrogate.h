@@ -44,15 +44,16 @@ int sur_gemm_bf16(const void *A, int lda, int a_kmajor, const void *B, int ldb, 
                   void *Yb, int M, int N, int K, const float *bias, int relu, int accumulate, void *stream);
 
 /*
- * The kernels behind sur_gemm_bf16.  With both operands K-major, lda and ldb
- * multiples of 8 and A, B 16-byte aligned, the product runs on the
- * fifth-generation tensor cores (tcgen05.mma, accumulator in tensor memory,
- * operands staged by TMA, 128 x 128 output tiles); any other layout on the
- * warp-level mma.sync kernel.  sur_gemm_set_path(p) selects for later calls
+ * The kernels behind sur_gemm_bf16.  With lda and ldb multiples of 8 and A, B
+ * 16-byte aligned the product runs on the fifth-generation tensor cores
+ * (tcgen05.mma, accumulator in tensor memory, operands staged by TMA, 128 x 128
+ * output tiles; either operand K-major or transposed); other strides and base
+ * addresses on the warp-level mma.sync kernel.  sur_gemm_set_path(p) selects for later calls
  * (process-wide): 0 that automatic choice (the default), 1 mma.sync always,
  * 2 tcgen05 with 128-byte swizzled operand slices only, 3 tcgen05 with
- * unswizzled core-matrix slices only (K a multiple of 8); with 2 or 3 a
- * product the tcgen05 kernel cannot take returns FDTD_ERR_ARG.
+ * unswizzled core-matrix slices only (K a multiple of 8); 2 and 3 take both
+ * operands K-major and return FDTD_ERR_ARG for a product their kernel cannot
+ * run.
  * sur_gemm_tc_launches: launches of the tcgen05 kernel so far.
  * sur_gemm_tc_failed: synchronises the device and returns 1 if a bounded
  * pipeline wait of the tcgen05 kernel gave up since the last call (that

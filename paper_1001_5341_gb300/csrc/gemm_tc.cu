@@ -1,5 +1,5 @@
 // gemm_tc.cu -- the surrogate's bf16 GEMM on the fifth-generation tensor
-// cores (surrogate.h: sur_gemm_bf16 with both operands K-major, and
+// cores (surrogate.h: sur_gemm_bf16, either operand K-major or transposed, and
 // sur_gemm_bf16_batched).
 //
 // Output tiles of 128 x 128, f32 accumulators in tensor memory, operands
@@ -10,11 +10,13 @@
 // columns per warp) and stored through a 32 x 33 transpose tile in shared
 // memory, so that each row is written by 32 lanes together, with the fused
 // epilogue (row scale, accumulate, bias, ReLU, f32 store and bf16 copy).
-// Two kernels:
+// Three kernels:
 //   k_gemm_tcp (128-byte swizzled 64-element K slices, the default):
 //     persistent, two CTAs per SM, warp-specialised -- one thread loads, one
 //     issues MMAs into two accumulators in turn, four warps run the epilogue
 //     of the previous tile meanwhile (below);
+//   k_gemm_split (the same slices): few output tiles and a transposed operand,
+//     the K range split over a cluster of CTAs (below);
 //   k_gemm_tc<0> (unswizzled core-matrix slices, 8 x 16 bytes from a 3-D
 //     tensor map over (8 elements, rows, K / 8)): one CTA per tile, thread 0
 //     loads and issues, the four warps run the epilogue at the end.
@@ -24,6 +26,7 @@
 // (sur_gemm_tc_failed), stops, lets its MMAs and loads in flight complete and
 // frees its tensor memory.
 #include <cuda.h>
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -61,8 +64,8 @@ static_assert(2 * stage_bytes<0>() >= 4 * 32 * 33 * 4 && 2 * stage_bytes<1>() >=
               "transpose tiles fit in two stages");
 
 // instruction descriptor, kind::f16: D f32 (bits 4-5 = 1), A and B bf16
-// (bits 7-9, 10-12 = 1), both K-major (bits 15, 16 = 0), N >> 3 at bit 17,
-// M >> 4 at bit 24
+// (bits 7-9, 10-12 = 1), both K-major (bits 15, 16 = 0; 1: MN-major), N >> 3 at
+// bit 17, M >> 4 at bit 24
 constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
                            ((uint32_t)(BM >> 4) << 24);
 
@@ -133,7 +136,65 @@ struct Epi {
     int ldy, relu, accumulate;
     int a3, b3;   // A, B tensor maps carry a batch dimension (else shared by the batch)
     int ystore;   // the persistent kernel stores Y by TMA (no accumulate, no bf16 copy)
+    int amn, bmn; // A, B MN-major (transposed: consecutive M or N)
 };
+
+// 128-byte-swizzled slices of 64 K by 128 rows of an operand.  K-major: one
+// box of 128 rows x 64 K; a step of 16 K is 32 bytes further along the rows,
+// groups of 8 rows are 1024 bytes apart.  MN-major: two boxes of 64 K rows x 64
+// consecutive M (or N), 8 KB apart; a step of 16 K is 16 rows (2 KB) further,
+// groups of 8 K rows 1024 bytes apart.
+__device__ __forceinline__ uint64_t operand_desc(uint32_t a, int k, int mn) {
+    return mn ? mdesc(a + 2048u * k, 8192u, 1024u, 2u) : mdesc(a + 32u * k, 16u, 1024u, 2u);
+}
+__device__ __forceinline__ void load_operand(unsigned char *dst, const CUtensorMap *m, uint64_t *bar, int mn, int d3,
+                                             int k0, int r0, int b) {
+    if (mn) {
+        tma_load2(dst, m, bar, r0, k0);
+        tma_load2(dst + 8192, m, bar, r0 + 64, k0);
+    } else if (d3) {
+        tma_load3b(dst, m, bar, k0, r0, b);
+    } else {
+        tma_load2(dst, m, bar, k0, r0);
+    }
+}
+__device__ __forceinline__ uint32_t idesc_of(const Epi &E) {
+    return IDESC | ((uint32_t)E.amn << 15) | ((uint32_t)E.bmn << 16);
+}
+
+// One element of the epilogue
+__device__ __forceinline__ void finish(const Epi &E, float *Yz, unsigned short *Ybz, int row, int n, float v) {
+    const long long o = (long long)row * E.ldy + n;
+    if (E.row_scale) v *= E.alpha * E.row_scale[row];
+    else if (E.alpha != 1.f) v *= E.alpha;
+    if (E.accumulate) v += Yz[o];
+    if (E.bias) v += E.bias[n];
+    if (E.relu) v = fmaxf(v, 0.f);
+    Yz[o] = v;
+    if (Ybz) Ybz[o] = __bfloat16_as_ushort(__float2bfloat16_rn(v));
+}
+
+// The same of four columns (16-byte aligned rows of Y, 8-byte of Yb)
+__device__ __forceinline__ void finish4(const Epi &E, int row, int n, float4 v) {
+    const long long o = (long long)row * E.ldy + n;
+    const float sc = E.row_scale ? E.alpha * E.row_scale[row] : E.alpha;
+    if (sc != 1.f) v = make_float4(v.x * sc, v.y * sc, v.z * sc, v.w * sc);
+    float *e = reinterpret_cast<float *>(&v);
+    if (E.accumulate) {
+        const float4 y = *reinterpret_cast<const float4 *>(E.Y + o);
+        v = make_float4(v.x + y.x, v.y + y.y, v.z + y.z, v.w + y.w);
+    }
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        if (E.bias) e[t] += E.bias[n + t];
+        if (E.relu) e[t] = fmaxf(e[t], 0.f);
+    }
+    *reinterpret_cast<float4 *>(E.Y + o) = v;
+    if (E.Yb)
+        *reinterpret_cast<ushort4 *>(E.Yb + o) = make_ushort4(
+            __bfloat16_as_ushort(__float2bfloat16_rn(v.x)), __bfloat16_as_ushort(__float2bfloat16_rn(v.y)),
+            __bfloat16_as_ushort(__float2bfloat16_rn(v.z)), __bfloat16_as_ushort(__float2bfloat16_rn(v.w)));
+}
 
 template <int SW>
 __global__ void __launch_bounds__(NT, 1) k_gemm_tc(const __grid_constant__ CUtensorMap ma,
@@ -367,16 +428,15 @@ __global__ void __launch_bounds__(PNT, 1) k_gemm_tcp(const __grid_constant__ CUt
                     }
                     unsigned char *a = sm + s * stage_bytes<1>();
                     mbar_expect_tx(&full[s], (uint32_t)stage_bytes<1>());
-                    if (E.a3) tma_load3b(a, &ma, &full[s], c * BK, m0, b);
-                    else tma_load2(a, &ma, &full[s], c * BK, m0);
-                    if (E.b3) tma_load3b(a + a_bytes<1>(), &mb, &full[s], c * BK, n0, b);
-                    else tma_load2(a + a_bytes<1>(), &mb, &full[s], c * BK, n0);
+                    load_operand(a, &ma, &full[s], E.amn, E.a3, c * BK, m0, b);
+                    load_operand(a + a_bytes<1>(), &mb, &full[s], E.bmn, E.b3, c * BK, n0, b);
                 }
             }
             s_issued = it;
         }
     } else if (warp == 5) {
         if (lane == 0) {   // MMA issuer
+            const uint32_t idesc = idesc_of(E);
             int it = 0, lt = 0;
             for (int t = blockIdx.x; t < total_tiles && !*fail; t += gridDim.x, ++lt) {
                 const int buf = lt & 1;
@@ -397,8 +457,7 @@ __global__ void __launch_bounds__(PNT, 1) k_gemm_tcp(const __grid_constant__ CUt
                     const uint32_t a0 = sa(sm + s * stage_bytes<1>()), b0 = a0 + a_bytes<1>();
 #pragma unroll
                     for (int k = 0; k < KSTEPS; ++k)
-                        mma_f16(d, mdesc(a0 + 32u * k, 16u, 1024u, 2u), mdesc(b0 + 32u * k, 16u, 1024u, 2u), IDESC,
-                                (c | k) != 0);
+                        mma_f16(d, operand_desc(a0, k, E.amn), operand_desc(b0, k, E.bmn), idesc, (c | k) != 0);
                     mma_commit(&empty[s]);
                 }
                 mma_commit(&acc_full[buf]);
@@ -516,6 +575,182 @@ __global__ void __launch_bounds__(PNT, 1) k_gemm_tcp(const __grid_constant__ CUt
     }
 }
 
+// ---- few output tiles, many K slices: the K range split over a cluster ----
+//
+// The weight gradients of the surrogate's layers are products of 64 .. 2048
+// rows and columns over thousands of K (dW = dz^T h): 1 to 128 tiles of the
+// persistent kernel, one long march of K slices each.  Here a cluster of S CTAs
+// (one per SM) takes an output tile, each CTA a share of the K slices in a ring
+// of up to six stages; every CTA's partial tile goes to its shared memory and
+// each CTA adds the S partials of 128 / S rows through distributed shared
+// memory, in rank order, and finishes them.  Bound by the latency of a share's
+// slices.  1024 x 1024 x 4096 (both operands MN-major): 27.8 us; mma.sync
+// 564 us.
+constexpr int SNS = 6;          // most stages
+constexpr int SMAX = 8;         // CTAs of a cluster (the portable size)
+__host__ __device__ constexpr int ssmem_bytes() { return 1024 + SNS * stage_bytes<1>() + 256; }
+static_assert(2 * stage_bytes<1>() >= BM * BN * 4, "a partial tile fits in two stages");
+
+__global__ void __launch_bounds__(NT, 1) k_gemm_split(const __grid_constant__ CUtensorMap ma,
+                                                      const __grid_constant__ CUtensorMap mb, const Epi E, int M,
+                                                      int N, int K, int S) {
+    namespace cg = cooperative_groups;
+    constexpr int BK = Cfg<1>::BK, KSTEPS = BK / 16;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char *sm = smem_raw + ((1024u - (sa(smem_raw) & 1023u)) & 1023u);
+    uint64_t *full = reinterpret_cast<uint64_t *>(sm + SNS * stage_bytes<1>());
+    uint64_t *empty = full + SNS;
+    uint64_t *done = empty + SNS;
+    uint32_t *tholder = reinterpret_cast<uint32_t *>(done + 1);
+    __shared__ int s_ok;
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = blockIdx.x % S, tile = blockIdx.x / S, tn = (N + BN - 1) / BN;
+    const int m0 = tile / tn * BM, n0 = tile % tn * BN;
+    const int slices = (K + BK - 1) / BK, share = (slices + S - 1) / S;
+    const int c0 = min(slices, rank * share), nk = min(slices, c0 + share) - c0;   // this CTA's slices
+
+    if (tid == 0) {
+        for (int s = 0; s < SNS; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(done, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        s_ok = 1;
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sa(tholder)),
+                     "r"(TMEM_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = *tholder;
+
+    if (tid == 0 && nk > 0) {
+        const uint32_t idesc = idesc_of(E);
+        auto issue = [&](int c) {
+            unsigned char *a = sm + c % SNS * stage_bytes<1>();
+            mbar_expect_tx(&full[c % SNS], (uint32_t)stage_bytes<1>());
+            load_operand(a, &ma, &full[c % SNS], E.amn, 0, (c0 + c) * BK, m0, 0);
+            load_operand(a + a_bytes<1>(), &mb, &full[c % SNS], E.bmn, 0, (c0 + c) * BK, n0, 0);
+        };
+        bool ok = true;
+        int issued = 0, c = 0;
+        for (; issued < SNS && issued < nk; ++issued) issue(issued);
+        for (; c < nk; ++c) {
+            const int s = c % SNS;
+            if (!mbar_wait(&full[s], (uint32_t)(c / SNS) & 1u)) {
+                ok = false;
+                break;
+            }
+            fence_after();
+            const uint32_t a0 = sa(sm + s * stage_bytes<1>()), b0 = a0 + a_bytes<1>();
+#pragma unroll
+            for (int k = 0; k < KSTEPS; ++k)
+                mma_f16(tmem, operand_desc(a0, k, E.amn), operand_desc(b0, k, E.bmn), idesc, (c | k) != 0);
+            mma_commit(&empty[s]);
+            // refill the stage of the slice before, whose MMAs have had a slice's time to finish
+            if (c >= 1 && issued < nk) {
+                if (!mbar_wait(&empty[(c - 1) % SNS], (uint32_t)((c - 1) / SNS) & 1u)) {
+                    ok = false;
+                    break;
+                }
+                issue(issued++);
+            }
+        }
+        mma_commit(done);   // completes once every MMA issued above has
+        if (!ok) {
+            atomicOr(&g_fail, 1);
+            s_ok = 0;
+            // let the loads in flight land before the CTA ends
+            for (int r = c + 1; r < issued; ++r) mbar_wait(&full[r % SNS], (uint32_t)(r / SNS) & 1u);
+        }
+    }
+    const bool dok = nk == 0 || mbar_wait(done, 0);
+    fence_after();
+    __syncthreads();
+    // this CTA's partial tile, row-major in the idle stage memory, the groups of
+    // four columns of a chunk permuted by the row so that neither side conflicts
+    float *part = reinterpret_cast<float *>(sm);
+    const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
+#pragma unroll 1
+    for (int cc = 0; cc < BN; cc += 32) {
+        uint32_t r[32];
+        if (nk > 0) {
+            tmem_ld32(trow + (uint32_t)cc, r);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) r[j] = 0u;
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            sts4(part + (warp * 32 + lane) * BN + cc + 4 * (j ^ (lane & 7)),
+                 make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]), __uint_as_float(r[4 * j + 2]),
+                             __uint_as_float(r[4 * j + 3])));
+    }
+    if (!dok && tid == 0) {
+        atomicOr(&g_fail, 1);
+        s_ok = 0;
+    }
+    fence_before();
+    auto cluster = cg::this_cluster();
+    cluster.sync();
+    bool good = true;
+    for (int r = 0; r < S; ++r) good = good && *cluster.map_shared_rank(&s_ok, r) != 0;
+    if (good) {
+        // a lane: four columns of a row of the S partial tiles, four rows at a time
+        const int col = n0 + 4 * lane, rows = BM / S;   // rows: a multiple of 16
+        const bool vec = col + 3 < N && E.ldy % 4 == 0 && (reinterpret_cast<uintptr_t>(E.Y) & 15) == 0 &&
+                         (reinterpret_cast<uintptr_t>(E.Yb) & 7) == 0;
+        for (int r0 = rank * rows + 4 * warp; r0 < (rank + 1) * rows; r0 += 16) {
+            float4 v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int r = 0; r < S; ++r) {
+                const float *q = cluster.map_shared_rank(part, r);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int lr = r0 + u;
+                    const float4 x = lds4(q + lr * BN + (lane & ~7) * 4 + 4 * ((lane & 7) ^ (lr & 7)));
+                    v[u].x += x.x; v[u].y += x.y; v[u].z += x.z; v[u].w += x.w;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int row = m0 + r0 + u;
+                if (row >= M) continue;
+                if (vec) {
+                    finish4(E, row, col, v[u]);
+                } else {
+                    const float e[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+                    for (int t = 0; t < 4; ++t)
+                        if (col + t < N) finish(E, E.Y, E.Yb, row, col + t, e[t]);
+                }
+            }
+        }
+    }
+    cluster.sync();   // a CTA's partial tile stays until every CTA has read it
+    if (warp == 0) {
+        fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+    }
+}
+
+// MN-major operand: rows consecutive, K rows ld apart
+bool encode_mnmajor(EncodeTiled enc, CUtensorMap *m, const void *p, int rows, int K, int ld) {
+    cuuint64_t dims[2] = {(cuuint64_t)rows, (cuuint64_t)K};
+    cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
+    cuuint32_t box[2] = {64, 64}, es[2] = {1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(p), dims, strides, box, es,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // batch > 1 with stride > 0 (elements): a third dimension over the batch
 bool encode_kmajor(EncodeTiled enc, CUtensorMap *m, const void *p, int rows, int K, int ld, int box_rows, int sw,
                    int batch = 1, long long stride = 0) {
@@ -546,13 +781,13 @@ long long g_launches = 0;       // launches of k_gemm_tc
 
 int tc_path() { return g_path; }
 
-// Whether (and how) the tcgen05 kernel runs this product: 1 (128-byte
-// swizzle), 0 (core matrices), -1 (it cannot: sur_gemm_bf16 runs mma.sync).
+// Whether (and how) the tcgen05 kernels run this product: 1 (128-byte
+// swizzle), 0 (core matrices), -1 (they cannot: sur_gemm_bf16 runs mma.sync).
+// Transposed (MN-major) operands only by the automatic choice.
 int tc_layout(const void *A, int lda, int a_kmajor, const void *B, int ldb, int b_kmajor, int K) {
     if (g_path == 1) return -1;
-    const bool kmajor = a_kmajor && b_kmajor && lda % 8 == 0 && ldb % 8 == 0 &&
-                        (reinterpret_cast<uintptr_t>(A) & 15) == 0 && (reinterpret_cast<uintptr_t>(B) & 15) == 0;
-    if (!kmajor) return -1;
+    if (lda % 8 || ldb % 8 || (reinterpret_cast<uintptr_t>(A) & 15) || (reinterpret_cast<uintptr_t>(B) & 15)) return -1;
+    if (!(a_kmajor && b_kmajor)) return g_path == 0 ? 1 : -1;
     if (g_path == 3) return K % 8 == 0 ? 0 : -1;
     return 1;
 }
@@ -561,7 +796,7 @@ namespace {
 // launch of k_gemm_tc over batch products (layout 1 only when batch > 1)
 int launch_tc(int layout, const void *A, int lda, long long sa, const void *B, int ldb, long long sb, int batch,
               Epi E, int M, int N, int K, cudaStream_t s) {
-    static bool attr_set[2] = {false, false};
+    static bool attr_set[3] = {false, false, false};
     EncodeTiled enc = encoder();
     if (!enc) return FDTD_ERR_CUDA;
     CUtensorMap ma, mb, my;
@@ -580,11 +815,33 @@ int launch_tc(int layout, const void *A, int lda, long long sa, const void *B, i
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     }
     if (!E.ystore) std::memset(&my, 0, sizeof(my));   // unused
-    if (!encode_kmajor(enc, &ma, A, M, K, lda, BM, layout, batch, sa) ||
-        !encode_kmajor(enc, &mb, B, N, K, ldb, BN, layout, batch, sb))
+    if (!(E.amn ? encode_mnmajor(enc, &ma, A, M, K, lda) : encode_kmajor(enc, &ma, A, M, K, lda, BM, layout, batch, sa)) ||
+        !(E.bmn ? encode_mnmajor(enc, &mb, B, N, K, ldb) : encode_kmajor(enc, &mb, B, N, K, ldb, BN, layout, batch, sb)))
         return FDTD_ERR_CUDA;
     cudaError_t e = cudaSuccess;
-    if (layout == 1) {
+    const long long out_tiles = (long long)((N + BN - 1) / BN) * ((M + BM - 1) / BM);
+    const int slices = (K + Cfg<1>::BK - 1) / Cfg<1>::BK;
+    if (layout == 1 && (E.amn || E.bmn) && out_tiles <= 128) {
+        // tiles for less than one CTA per SM: split K while the CTAs fit one per
+        // SM and a share has four slices or more
+        int S = 1;
+        while (S < SMAX && out_tiles * S * 2 <= 152 && slices / (2 * S) >= 4) S *= 2;
+        if (!attr_set[2])
+            e = cudaFuncSetAttribute(k_gemm_split, cudaFuncAttributeMaxDynamicSharedMemorySize, ssmem_bytes());
+        attr_set[2] = e == cudaSuccess;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)(out_tiles * S));
+        cfg.blockDim = dim3(NT);
+        cfg.dynamicSmemBytes = ssmem_bytes();
+        cfg.stream = s;
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = S;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, k_gemm_split, ma, mb, E, M, N, K, S);
+    } else if (layout == 1) {
         // persistent: two CTAs per SM over all output tiles of the batch
         static int sms = 0;
         if (sms == 0) {
@@ -617,8 +874,8 @@ int launch_tc(int layout, const void *A, int lda, long long sa, const void *B, i
 }
 }  // namespace
 
-int gemm_tc(int layout, const void *A, int lda, const void *B, int ldb, float *Y, int ldy, void *Yb, int M, int N,
-            int K, const float *bias, int relu, int accumulate, cudaStream_t s) {
+int gemm_tc(int layout, const void *A, int lda, int a_kmajor, const void *B, int ldb, int b_kmajor, float *Y, int ldy,
+            void *Yb, int M, int N, int K, const float *bias, int relu, int accumulate, cudaStream_t s) {
     Epi E;
     E.Y = Y;
     E.sy = 0;
@@ -629,6 +886,8 @@ int gemm_tc(int layout, const void *A, int lda, const void *B, int ldb, float *Y
     E.ldy = ldy;
     E.relu = relu;
     E.accumulate = accumulate;
+    E.amn = !a_kmajor;
+    E.bmn = !b_kmajor;
     return launch_tc(layout, A, lda, 0, B, ldb, 0, 1, E, M, N, K, s);
 }
 
@@ -664,6 +923,7 @@ int sur_gemm_bf16_batched(const void *A, int lda, long long sa, const void *B, i
     E.ldy = ldy;
     E.relu = 0;
     E.accumulate = 0;
+    E.amn = E.bmn = 0;
     return launch_tc(1, A, lda, sa, B, ldb, sb, batch, E, M, N, K, static_cast<cudaStream_t>(stream));
 }
 

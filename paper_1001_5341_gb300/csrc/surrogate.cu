@@ -1,14 +1,15 @@
 // surrogate.cu -- forward/backward kernels and the optimiser step of the
 // learned near-field surrogate (declarations and contracts: surrogate.h).
 //
-// The GEMM with both operands K-major (and 16-byte rows) runs on the
-// fifth-generation tensor cores (tcgen05, TMEM, TMA: gemm_tc.cu).  The other
-// operand layouts run on the warp-level mma.sync m16n8k16 bf16 instruction:
+// The GEMM with 16-byte operand rows runs on the fifth-generation tensor cores
+// (tcgen05, TMEM, TMA: gemm_tc.cu).  Other row strides and base addresses run on
+// the warp-level mma.sync m16n8k16 bf16 instruction:
 // 64x64 block tiles, 32-deep k slices staged in shared memory (either operand
 // layout, transposed while staging), four warps of 32x32, f32 accumulators,
 // fused bias / ReLU / bf16-copy epilogue.  The
 // convolutions, the elementwise steps and the reductions are plain SIMT
 // kernels: they are a few percent of the network's arithmetic.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -205,28 +206,65 @@ __global__ void k_conv_bwd_x(const bf16raw *__restrict__ w, const float *__restr
 
 // ---- elementwise and reductions ------------------------------------------------
 
-__global__ void k_relu_bwd(const float *y, const float *dy, float *dz, bf16raw *dzb, long long n) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const float v = y[i] > 0.f ? dy[i] : 0.f;
-        dz[i] = v;
-        if (dzb) dzb[i] = tobf(v);
+// V: elements a thread moves at once (4: float4 and 8-byte bf16 accesses)
+template <int V>
+__global__ void k_relu_bwd(const float *__restrict__ y, const float *__restrict__ dy, float *dz, bf16raw *dzb,
+                           long long n) {
+    const long long step = (long long)gridDim.x * blockDim.x * V;
+    for (long long i = (blockIdx.x * (long long)blockDim.x + threadIdx.x) * V; i < n; i += step) {
+        if constexpr (V == 4) {
+            const float4 a = *reinterpret_cast<const float4 *>(y + i), d = *reinterpret_cast<const float4 *>(dy + i);
+            const float4 v = make_float4(a.x > 0.f ? d.x : 0.f, a.y > 0.f ? d.y : 0.f, a.z > 0.f ? d.z : 0.f,
+                                         a.w > 0.f ? d.w : 0.f);
+            *reinterpret_cast<float4 *>(dz + i) = v;
+            if (dzb) *reinterpret_cast<ushort4 *>(dzb + i) = make_ushort4(tobf(v.x), tobf(v.y), tobf(v.z), tobf(v.w));
+        } else {
+            const float v = y[i] > 0.f ? dy[i] : 0.f;
+            dz[i] = v;
+            if (dzb) dzb[i] = tobf(v);
+        }
     }
 }
 
-// one block per 32 columns: a warp per column stripe, threads over rows
-__global__ void k_bias_grad(const float *dz, int ldz, int M, int N, float *db) {
-    __shared__ float red[8][33];
-    const int col = blockIdx.x * 32 + (threadIdx.x & 31), ry = threadIdx.x >> 5;
+// Column sums.  A cluster of up to eight blocks takes 32 columns, each block a
+// share of the rows, 32 warps over its rows with eight loads in flight; the
+// blocks' sums meet in distributed shared memory in rank order.  (One block of
+// eight warps per 32 columns: 41 us on 4096 x 1024, latency bound; now 7.8 us.)
+constexpr int BG_W = 32;
+__global__ void __launch_bounds__(32 * BG_W) k_bias_grad(const float *__restrict__ dz, int ldz, int M, int N, float *db,
+                                                         int S) {
+    namespace cg = cooperative_groups;
+    __shared__ float red[BG_W][33], sum[32];
+    const int rank = blockIdx.x % S, lane = threadIdx.x & 31, ry = threadIdx.x >> 5;
+    const int col = blockIdx.x / S * 32 + lane;
+    const int share = (M + S - 1) / S, m0 = min(M, rank * share), m1 = min(M, m0 + share);
     float s = 0.f;
-    if (col < N)
-        for (int m = ry; m < M; m += 8) s += dz[(long long)m * ldz + col];
-    red[ry][threadIdx.x & 31] = s;
+    if (col < N) {
+        const float *p = dz + col;
+        int m = m0 + ry;
+        for (; m + 7 * BG_W < m1; m += 8 * BG_W) {
+            float v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = p[(long long)(m + u * BG_W) * ldz];
+            s += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+        }
+        for (; m < m1; m += BG_W) s += p[(long long)m * ldz];
+    }
+    red[ry][lane] = s;
     __syncthreads();
-    if (ry == 0 && col < N) {
+    if (ry == 0) {
         float t = 0.f;
-        for (int r = 0; r < 8; ++r) t += red[r][threadIdx.x & 31];
+        for (int r = 0; r < BG_W; ++r) t += red[r][lane];
+        sum[lane] = t;
+    }
+    auto cluster = cg::this_cluster();
+    cluster.sync();
+    if (rank == 0 && ry == 0 && col < N) {
+        float t = 0.f;
+        for (int r = 0; r < S; ++r) t += cluster.map_shared_rank(sum, r)[lane];
         db[col] = t;
     }
+    cluster.sync();
 }
 
 __global__ void k_cast(const float *x, bf16raw *y, long long n) {
@@ -383,6 +421,8 @@ __global__ void k_assemble_bwd(const float *__restrict__ dout, const float *__re
     }
 }
 
+bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
 int grid_for(long long n, int threads) {
     long long b = (n + threads - 1) / threads;
     if (b > 4096) b = 4096;
@@ -512,8 +552,8 @@ namespace gtc {
 // path selected by sur_gemm_set_path, and its launch
 int tc_layout(const void *A, int lda, int a_kmajor, const void *B, int ldb, int b_kmajor, int K);
 int tc_path();
-int gemm_tc(int layout, const void *A, int lda, const void *B, int ldb, float *Y, int ldy, void *Yb, int M, int N,
-            int K, const float *bias, int relu, int accumulate, cudaStream_t s);
+int gemm_tc(int layout, const void *A, int lda, int a_kmajor, const void *B, int ldb, int b_kmajor, float *Y, int ldy,
+            void *Yb, int M, int N, int K, const float *bias, int relu, int accumulate, cudaStream_t s);
 }  // namespace gtc
 }  // namespace fdtd
 
@@ -524,9 +564,11 @@ int sur_gemm_bf16(const void *A, int lda, int a_kmajor, const void *B, int ldb, 
     if (!A || !B || !Y || M < 1 || N < 1 || K < 1 || lda < 1 || ldb < 1 || ldy < N) return FDTD_ERR_ARG;
     if ((a_kmajor ? lda < K : lda < M) || (b_kmajor ? ldb < K : ldb < N)) return FDTD_ERR_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // both operands K-major with 16-byte rows: the tcgen05 kernel; else mma.sync
+    // operands with 16-byte rows: the tcgen05 kernels; else mma.sync
     const int layout = fdtd::gtc::tc_layout(A, lda, a_kmajor, B, ldb, b_kmajor, K);
-    if (layout >= 0) return fdtd::gtc::gemm_tc(layout, A, lda, B, ldb, Y, ldy, Yb, M, N, K, bias, relu, accumulate, s);
+    if (layout >= 0) 
+        return fdtd::gtc::gemm_tc(layout, A, lda, a_kmajor, B, ldb, b_kmajor, Y, ldy, Yb, M, N, K, bias, relu, accumulate,
+                                  s);
     if (fdtd::gtc::tc_path() >= 2) return FDTD_ERR_ARG;   // the tcgen05 kernel alone was asked for
     const dim3 grid((N + GBN - 1) / GBN, (M + GBM - 1) / GBM);
     const bf16raw *a = static_cast<const bf16raw *>(A), *b = static_cast<const bf16raw *>(B);
@@ -575,15 +617,35 @@ int sur_conv1d_bwd(const float *x, int xs, const void *w, const float *y, const 
 
 int sur_relu_bwd(const float *y, const float *dy, float *dz, void *dzb, long long n, void *stream) {
     if (!y || !dy || !dz || n < 1) return FDTD_ERR_ARG;
-    k_relu_bwd<<<grid_for(n, 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(y, dy, dz,
-                                                                                  static_cast<bf16raw *>(dzb), n);
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    bf16raw *zb = static_cast<bf16raw *>(dzb);
+    // 16-byte accesses where every array allows them (4096 x 1024: 18.5 us scalar, 8.9 us)
+    if (n % 4 == 0 && aligned16(y) && aligned16(dy) && aligned16(dz) && (reinterpret_cast<uintptr_t>(dzb) & 7) == 0)
+        k_relu_bwd<4><<<grid_for(n / 4, 256), 256, 0, s>>>(y, dy, dz, zb, n);
+    else
+        k_relu_bwd<1><<<grid_for(n, 256), 256, 0, s>>>(y, dy, dz, zb, n);
     return launched();
 }
 
 int sur_bias_grad(const float *dz, int ldz, int M, int N, float *db, void *stream) {
     if (!dz || !db || M < 1 || N < 1 || ldz < N) return FDTD_ERR_ARG;
-    k_bias_grad<<<(N + 31) / 32, 256, 0, static_cast<cudaStream_t>(stream)>>>(dz, ldz, M, N, db);
-    return launched();
+    int S = 1;   // blocks per 32 columns: while they fit two per SM and have 256 rows or more each
+    while (S < 8 && (long long)((N + 31) / 32) * S * 2 <= 2 * 152 && M / (2 * S) >= 256) S *= 2;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)((N + 31) / 32 * S));
+    cfg.blockDim = dim3(32 * BG_W);
+    cfg.stream = static_cast<cudaStream_t>(stream);
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = S;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, k_bias_grad, dz, ldz, M, N, db, S) != cudaSuccess) {
+        cudaGetLastError();
+        return FDTD_ERR_CUDA;
+    }
+    return FDTD_OK;
 }
 
 int sur_cast_bf16(const float *x, void *y, long long n, void *stream) {
