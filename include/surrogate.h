@@ -232,6 +232,24 @@ int sur_lattice_weights_kmajor(const void *G, const int *ant, int A, int K, int 
    [rows][ld], ld >= 3K: the A operand of [hi, hi, lo] [W_hi; W_lo; W_hi]. */
 int sur_split3_bf16(const float *x, int rows, int K, void *out, int ld, void *stream);
 
+/*
+ * Every profile at every antenna, in three launches: the traces
+ *   out[a][p][t] = c_out peak_p sum_k (q[p][k] / peak_p) (Ghi + Glo)[ir_a][m_a - k + moff][t - S k + J]
+ * (peak_p = max |q[p]|; entries off the table are 0), f32 [A][P][T], as one
+ * batched tcgen05 GEMM of the split profiles [hi, hi, lo] with each antenna's
+ * weights [W_hi; W_lo; W_hi] (f32 accumulation).
+ *   Ghi, Glo: bf16 [NR][D][T] (sur_split_bf16); q: f32 [P][K]; ant: int [A][2];
+ *   work: 16-byte aligned device memory of sur_lattice_serve_bytes(P, A, K, T)
+ *   bytes or more, scratch for the call (FDTD_ERR_ARG if smaller); A <= 65535.
+ * FDTD_ERR_ARG also while sur_gemm_set_path has selected mma.sync (1) or the
+ * unswizzled layout (3).  sur_lattice_serve_bytes returns FDTD_ERR_ARG for a
+ * size below 1.
+ */
+long long sur_lattice_serve_bytes(int P, int A, int K, int T);
+int sur_lattice_serve(const void *Ghi, const void *Glo, const float *q, const int *ant, int P, int A, int K, int NR,
+                      int D, int T, int S, int J, int moff, float c_out, void *work, long long work_bytes, float *out,
+                      void *stream);
+
 #ifdef __cplusplus
 }
 #endif

@@ -137,6 +137,7 @@ struct Epi {
     int a3, b3;   // A, B tensor maps carry a batch dimension (else shared by the batch)
     int ystore;   // the persistent kernel stores Y by TMA (no accumulate, no bf16 copy)
     int amn, bmn; // A, B MN-major (transposed: consecutive M or N)
+    int bwrap;    // B's K index starts again at 0 from this K on (0: never)
 };
 
 // 128-byte-swizzled slices of 64 K by 128 rows of an operand.  K-major: one
@@ -149,7 +150,10 @@ __device__ __forceinline__ uint64_t operand_desc(uint32_t a, int k, int mn) {
 }
 __device__ __forceinline__ void load_operand(unsigned char *dst, const CUtensorMap *m, uint64_t *bar, int mn, int d3,
                                              int k0, int r0, int b) {
-    if (mn) {
+    if (mn && d3) {
+        tma_load3b(dst, m, bar, r0, k0, b);
+        tma_load3b(dst + 8192, m, bar, r0 + 64, k0, b);
+    } else if (mn) {
         tma_load2(dst, m, bar, r0, k0);
         tma_load2(dst + 8192, m, bar, r0 + 64, k0);
     } else if (d3) {
@@ -429,7 +433,8 @@ __global__ void __launch_bounds__(PNT, 1) k_gemm_tcp(const __grid_constant__ CUt
                     unsigned char *a = sm + s * stage_bytes<1>();
                     mbar_expect_tx(&full[s], (uint32_t)stage_bytes<1>());
                     load_operand(a, &ma, &full[s], E.amn, E.a3, c * BK, m0, b);
-                    load_operand(a + a_bytes<1>(), &mb, &full[s], E.bmn, E.b3, c * BK, n0, b);
+                    load_operand(a + a_bytes<1>(), &mb, &full[s], E.bmn, E.b3,
+                                 E.bwrap && c * BK >= E.bwrap ? c * BK - E.bwrap : c * BK, n0, b);
                 }
             }
             s_issued = it;
@@ -741,12 +746,14 @@ __global__ void __launch_bounds__(NT, 1) k_gemm_split(const __grid_constant__ CU
     }
 }
 
-// MN-major operand: rows consecutive, K rows ld apart
-bool encode_mnmajor(EncodeTiled enc, CUtensorMap *m, const void *p, int rows, int K, int ld) {
-    cuuint64_t dims[2] = {(cuuint64_t)rows, (cuuint64_t)K};
-    cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-    cuuint32_t box[2] = {64, 64}, es[2] = {1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(p), dims, strides, box, es,
+// MN-major operand: rows consecutive, K rows ld apart (and a batch as above)
+bool encode_mnmajor(EncodeTiled enc, CUtensorMap *m, const void *p, int rows, int K, int ld, int batch = 1,
+                    long long stride = 0) {
+    const int nd = batch > 1 && stride > 0 ? 3 : 2;
+    cuuint64_t dims[3] = {(cuuint64_t)rows, (cuuint64_t)K, (cuuint64_t)batch};
+    cuuint64_t strides[2] = {(cuuint64_t)ld * 2, (cuuint64_t)stride * 2};
+    cuuint32_t box[3] = {64, 64, 1}, es[3] = {1, 1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, nd, const_cast<void *>(p), dims, strides, box, es,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -815,13 +822,16 @@ int launch_tc(int layout, const void *A, int lda, long long sa, const void *B, i
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     }
     if (!E.ystore) std::memset(&my, 0, sizeof(my));   // unused
-    if (!(E.amn ? encode_mnmajor(enc, &ma, A, M, K, lda) : encode_kmajor(enc, &ma, A, M, K, lda, BM, layout, batch, sa)) ||
-        !(E.bmn ? encode_mnmajor(enc, &mb, B, N, K, ldb) : encode_kmajor(enc, &mb, B, N, K, ldb, BN, layout, batch, sb)))
+    const int KB = E.bwrap ? E.bwrap : K;   // K rows of B
+    if (!(E.amn ? encode_mnmajor(enc, &ma, A, M, K, lda, batch, sa)
+                : encode_kmajor(enc, &ma, A, M, K, lda, BM, layout, batch, sa)) ||
+        !(E.bmn ? encode_mnmajor(enc, &mb, B, N, KB, ldb, batch, sb)
+                : encode_kmajor(enc, &mb, B, N, KB, ldb, BN, layout, batch, sb)))
         return FDTD_ERR_CUDA;
     cudaError_t e = cudaSuccess;
     const long long out_tiles = (long long)((N + BN - 1) / BN) * ((M + BM - 1) / BM);
     const int slices = (K + Cfg<1>::BK - 1) / Cfg<1>::BK;
-    if (layout == 1 && (E.amn || E.bmn) && out_tiles <= 128) {
+    if (layout == 1 && (E.amn || E.bmn) && batch == 1 && !E.bwrap && out_tiles <= 128) {
         // tiles for less than one CTA per SM: split K while the CTAs fit one per
         // SM and a share has four slices or more
         int S = 1;
@@ -888,7 +898,28 @@ int gemm_tc(int layout, const void *A, int lda, int a_kmajor, const void *B, int
     E.accumulate = accumulate;
     E.amn = !a_kmajor;
     E.bmn = !b_kmajor;
+    E.bwrap = 0;
     return launch_tc(layout, A, lda, 0, B, ldb, 0, 1, E, M, N, K, s);
+}
+
+// The lattice surrogate's serving product: Y[a] = alpha diag(row_scale) Q W[a],
+// Q [M][3 KS] = [hi, hi, lo] K-major, W[a] [2 KS][ldw] = [W_hi; W_lo] with N
+// consecutive (so W_hi is read again for lo); KS a multiple of 64.
+int serve_gemm(const void *Q, const void *W, int ldw, float *Y, int M, int N, int KS, int batch, const float *row_scale,
+               float alpha, cudaStream_t s) {
+    if (g_path == 1 || g_path == 3) return FDTD_ERR_ARG;
+    Epi E;
+    E.Y = Y;
+    E.sy = (long long)M * N;
+    E.Yb = nullptr;
+    E.bias = nullptr;
+    E.row_scale = row_scale;
+    E.alpha = alpha;
+    E.ldy = N;
+    E.relu = E.accumulate = E.amn = 0;
+    E.bmn = 1;
+    E.bwrap = 2 * KS;
+    return launch_tc(1, Q, 3 * KS, 0, W, ldw, 2LL * KS * ldw, batch, E, M, N, 3 * KS, s);
 }
 
 }  // namespace gtc
@@ -923,7 +954,7 @@ int sur_gemm_bf16_batched(const void *A, int lda, long long sa, const void *B, i
     E.ldy = ldy;
     E.relu = 0;
     E.accumulate = 0;
-    E.amn = E.bmn = 0;
+    E.amn = E.bmn = E.bwrap = 0;
     return launch_tc(1, A, lda, sa, B, ldb, sb, batch, E, M, N, K, static_cast<cudaStream_t>(stream));
 }
 

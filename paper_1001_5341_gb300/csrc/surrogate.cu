@@ -544,6 +544,85 @@ __global__ void k_split3_bf16(const float *__restrict__ x, int rows, int K, bf16
     }
 }
 
+// ---- serving every profile at every antenna (sur_lattice_serve) ----
+
+// One warp per profile: its peak s, and the split of the normalised profile as
+// the A operand [hi, hi, lo], each part KS columns (zeros past K).
+__global__ void k_serve_profiles(const float *__restrict__ q, int P, int K, int KS, bf16raw *__restrict__ out,
+                                 float *__restrict__ s) {
+    const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (row >= P) return;
+    const float *qr = q + (long long)row * K;
+    float m = 0.f;
+    for (int i = lane; i < K; i += 32) m = fmaxf(m, fabsf(qr[i]));
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    const float inv = m > 0.f ? 1.f / m : 0.f;
+    bf16raw *o = out + (long long)row * 3 * KS;
+    for (int i = lane; i < KS; i += 32) {
+        const float x = i < K ? qr[i] * inv : 0.f;
+        const bf16raw h = tobf(x);
+        o[i] = o[KS + i] = h;
+        o[2 * KS + i] = tobf(x - bf(h));
+    }
+    if (lane == 0) s[row] = m;
+}
+
+// The B operands: W[a][k][t] = Ghi[ir][d][t - S k + J] for k < K, the same of Glo
+// from row KS, zeros where the table has no such entry.  A block copies rows k
+// (a warp each) of one antenna and part, eight t per lane: the table row is read
+// and W written along t, so both are coalesced (gathered K-major, two bytes a
+// lane along k, the same weights took 3 x 34.6 us for 64 antennas, now one launch of 10 us).
+// VEC: S, J and T are multiples of four and the tables 8-byte aligned, so that a
+// lane's eight entries are two 8-byte loads.
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_serve_weights(const bf16raw *__restrict__ Ghi, const bf16raw *__restrict__ Glo,
+                                                       const int *__restrict__ ant, int K, int KS, int NR, int D, int T,
+                                                       int TW, int S, int J, int moff, bf16raw *__restrict__ W) {
+    const int a = blockIdx.y, row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;   // row of 2 KS
+    const int k = row < KS ? row : row - KS;
+    const int ir = ant[2 * a], d = ant[2 * a + 1] - k + moff;
+    const bool on = k < K && ir >= 0 && ir < NR && d >= 0 && d < D;
+    const bf16raw *g = (row < KS ? Ghi : Glo) + ((long long)(on ? ir : 0) * D + (on ? d : 0)) * T;
+    bf16raw *w = W + ((long long)a * 2 * KS + row) * TW;
+    const int off = J - S * k;
+    for (int t = 8 * lane; t < TW; t += 256) {
+        ushort4 v[2] = {make_ushort4(0, 0, 0, 0), make_ushort4(0, 0, 0, 0)};
+        if (on) {
+            if (VEC) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int tau = t + 4 * h + off;   // a multiple of four: a quad lies inside the row or outside
+                    if (tau >= 0 && tau < T && t + 4 * h < T) v[h] = *reinterpret_cast<const ushort4 *>(g + tau);
+                }
+            } else {
+                bf16raw *e = reinterpret_cast<bf16raw *>(v);
+#pragma unroll
+                for (int h = 0; h < 8; ++h) {
+                    const int tau = t + h + off;
+                    if (tau >= 0 && tau < T && t + h < T) e[h] = g[tau];
+                }
+            }
+        }
+        *reinterpret_cast<uint4 *>(w + t) = *reinterpret_cast<const uint4 *>(v);
+    }
+}
+
+struct ServeLayout {
+    int KS, TW;                       // K rounded up to 64, T to 8
+    long long q, s, w, bytes;         // offsets of Q3, the peaks and W
+};
+ServeLayout serve_layout(int P, int A, int K, int T) {
+    ServeLayout L;
+    L.KS = (K + 63) / 64 * 64;
+    L.TW = (T + 7) / 8 * 8;
+    const auto up = [](long long n) { return (n + 255) / 256 * 256; };
+    L.q = 0;
+    L.s = up(2LL * P * 3 * L.KS);
+    L.w = L.s + up(4LL * P);
+    L.bytes = L.w + up(2LL * A * 2 * L.KS * L.TW);
+    return L;
+}
+
 }  // namespace
 
 namespace fdtd {
@@ -554,6 +633,8 @@ int tc_layout(const void *A, int lda, int a_kmajor, const void *B, int ldb, int 
 int tc_path();
 int gemm_tc(int layout, const void *A, int lda, int a_kmajor, const void *B, int ldb, int b_kmajor, float *Y, int ldy,
             void *Yb, int M, int N, int K, const float *bias, int relu, int accumulate, cudaStream_t s);
+int serve_gemm(const void *Q, const void *W, int ldw, float *Y, int M, int N, int KS, int batch, const float *row_scale,
+               float alpha, cudaStream_t s);
 }  // namespace gtc
 }  // namespace fdtd
 
@@ -787,6 +868,37 @@ int sur_lattice_weights(const void *G, const int *ant, int A, int K, int NR, int
     k_lat_weights<<<dim3((T + 255) / 256, K, A), 256, 0, static_cast<cudaStream_t>(stream)>>>(
         static_cast<const bf16raw *>(G), ant, K, NR, D, T, S, J, moff, static_cast<bf16raw *>(W));
     return launched();
+}
+
+long long sur_lattice_serve_bytes(int P, int A, int K, int T) {
+    if (P < 1 || A < 1 || K < 1 || T < 1) return FDTD_ERR_ARG;
+    return serve_layout(P, A, K, T).bytes;
+}
+
+int sur_lattice_serve(const void *Ghi, const void *Glo, const float *q, const int *ant, int P, int A, int K, int NR,
+                      int D, int T, int S, int J, int moff, float c_out, void *work, long long work_bytes, float *out,
+                      void *stream) {
+    if (!Ghi || !Glo || !q || !ant || !work || !out || P < 1 || A < 1 || A > 65535 || K < 1 || NR < 1 || D < 1 || T < 1 ||
+        S < 0 || J < 0 || !aligned16(work))
+        return FDTD_ERR_ARG;
+    const ServeLayout L = serve_layout(P, A, K, T);
+    if (work_bytes < L.bytes) return FDTD_ERR_ARG;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    char *w = static_cast<char *>(work);
+    bf16raw *Q = reinterpret_cast<bf16raw *>(w + L.q), *W = reinterpret_cast<bf16raw *>(w + L.w);
+    float *s = reinterpret_cast<float *>(w + L.s);
+    k_serve_profiles<<<(P + 7) / 8, 256, 0, st>>>(q, P, K, L.KS, Q, s);
+    const dim3 grid(2 * L.KS / 8, A);
+    const bf16raw *hi = static_cast<const bf16raw *>(Ghi), *lo = static_cast<const bf16raw *>(Glo);
+    const bool vec = S % 4 == 0 && J % 4 == 0 && T % 4 == 0 &&
+                     ((reinterpret_cast<uintptr_t>(Ghi) | reinterpret_cast<uintptr_t>(Glo)) & 7) == 0;
+    if (vec)
+        k_serve_weights<true><<<grid, 256, 0, st>>>(hi, lo, ant, K, L.KS, NR, D, T, L.TW, S, J, moff, W);
+    else
+        k_serve_weights<false><<<grid, 256, 0, st>>>(hi, lo, ant, K, L.KS, NR, D, T, L.TW, S, J, moff, W);
+    const int rc = launched();
+    if (rc != FDTD_OK) return rc;
+    return fdtd::gtc::serve_gemm(Q, W, L.TW, out, P, T, L.KS, A, s, c_out, st);
 }
 
 }  // extern "C"

@@ -35,9 +35,8 @@ import numpy as np
 
 from . import (check, fdtd_probes, profile_gaisser_hillas, lateral_nkg, Simulation, sur_adam, sur_antenna_features,
                sur_assemble, sur_assemble_bwd, sur_bias_grad, sur_cast_bf16, sur_gemm_bf16, sur_lattice_bwd,
-               sur_gemm_bf16_batched, sur_lattice_fwd, sur_lattice_fwd_f32, sur_lattice_weights,
-               sur_lattice_weights_kmajor, sur_mse,
-               sur_normalize_rows, sur_pairs, sur_relu_bwd, sur_scale_rows, sur_split3_bf16, sur_split_bf16)
+               sur_lattice_fwd, sur_lattice_fwd_f32, sur_lattice_serve, sur_lattice_serve_bytes, sur_mse,
+               sur_normalize_rows, sur_pairs, sur_relu_bwd, sur_scale_rows, sur_split_bf16)
 
 N_FEAT = 64
 
@@ -421,30 +420,19 @@ class Lattice:
     def predict_grid(self, q, ants):
         """Every profile q [P, K] at every antenna ants [A, 2]: traces
         [A, P, T]: one batched tensor-core GEMM (tcgen05: bf16 operands, f32
-        accumulation in tensor memory) of the split profiles [hi, hi, lo]
-        [P, 3K] with each antenna's K-major weights [W_hi; W_lo; W_hi]^T
-        [T, 3K], both padded to a row of KP = 3K rounded up to 8, the profile
-        scale applied in its epilogue."""
+        accumulation in tensor memory) of the split profiles [hi, hi, lo] with
+        each antenna's weights [W_hi; W_lo; W_hi], the profile scale applied in
+        its epilogue (sur_lattice_serve)."""
         import torch
         g = self.geo
-        P, A, K = q.shape[0], ants.shape[0], self.geo.K
-        KP = (3 * K + 7) // 8 * 8
-        st = _stream()
+        P, A = q.shape[0], ants.shape[0]
         if not self._split:
             self.split()
-        qn = torch.empty(P, K, dtype=torch.float32, device="cuda")
-        s = torch.empty(P, dtype=torch.float32, device="cuda")
-        check(sur_normalize_rows(_p(q), P, K, _p(qn), _p(s), st), "sur_normalize_rows")
-        Q3 = torch.empty(P, KP, dtype=torch.bfloat16, device="cuda")
-        check(sur_split3_bf16(_p(qn), P, K, _p(Q3), KP, st), "sur_split3_bf16")
-        W3 = torch.zeros(A, g.T, KP, dtype=torch.bfloat16, device="cuda")
-        for koff, tab in ((0, self.Ghi), (K, self.Glo), (2 * K, self.Ghi)):
-            check(sur_lattice_weights_kmajor(_p(tab), _p(ants), A, K, g.NR, self.D, g.T, g.S, g.J, self.moff, _p(W3),
-                                             KP, koff, st), "sur_lattice_weights_kmajor")
+        n = sur_lattice_serve_bytes(P, A, g.K, g.T)
+        work = torch.empty(n, dtype=torch.uint8, device="cuda")
         out = torch.empty(A, P, g.T, dtype=torch.float32, device="cuda")
-        # one launch for all antennas, the profile scale fused into the epilogue
-        check(sur_gemm_bf16_batched(_p(Q3), KP, 0, _p(W3), KP, g.T * KP, _p(out), g.T, P * g.T, P, g.T, KP, A, _p(s),
-                                    self.c_out, st), "sur_gemm_bf16_batched")
+        check(sur_lattice_serve(_p(self.Ghi), _p(self.Glo), _p(q), _p(ants), P, A, g.K, g.NR, self.D, g.T, g.S, g.J,
+                                self.moff, self.c_out, _p(work), n, _p(out), _stream()), "sur_lattice_serve")
         return out
 
 
