@@ -233,6 +233,26 @@ int sur_lattice_weights_kmajor(const void *G, const int *ant, int A, int K, int 
 int sur_split3_bf16(const float *x, int rows, int K, void *out, int ld, void *stream);
 
 /*
+ * One training step of the lattice table on B pairs (shower, antenna): the
+ * forward map of sur_lattice_fwd_f32 from the normalised profiles qn [B][K] with
+ * peaks s [B] (sur_normalize_rows), the mean squared error over all B T samples
+ * and its gradient, then the Adam update of G with moments m, v (sur_adam, step
+ * t >= 1).  Error terms of pair b:
+ *   st == NULL: y - target / (c_out s_b), target the traces [B][T];
+ *   else:       y c_out s_b / st_b - target, target the traces divided by their
+ *               own peaks st [B] (sur_normalize_rows).
+ * dG [NR][D][T] and dy [B][T] are overwritten with the gradients with respect to
+ * G and y, loss [1] with the loss.  work: 8-byte aligned device memory of
+ * sur_lattice_step_bytes(B, NR) bytes or more, scratch for the call.  B <= 65535,
+ * K <= 1024, NR <= 65534; FDTD_ERR_ARG otherwise.
+ */
+long long sur_lattice_step_bytes(int B, int NR);
+int sur_lattice_step(float *G, float *dG, float *m, float *v, const float *qn, const float *s, const int *ant,
+                     const float *target, const float *st, int B, int K, int NR, int D, int T, int S, int J, int moff,
+                     float c_out, float lr, float b1, float b2, float eps, int t, float *dy, float *loss, void *work,
+                     long long work_bytes, void *stream);
+
+/*
  * Every profile at every antenna, in three launches: the traces
  *   out[a][p][t] = c_out peak_p sum_k (q[p][k] / peak_p) (Ghi + Glo)[ir_a][m_a - k + moff][t - S k + J]
  * (peak_p = max |q[p]|; entries off the table are 0), f32 [A][P][T], as one

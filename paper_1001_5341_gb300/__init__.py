@@ -96,6 +96,9 @@ _SIGS = {
     "sur_lattice_weights": (_i, [_vp, _vp, _i, _i, _i, _i, _i, _i, _i, _i, _vp, _vp]),
     "sur_lattice_weights_kmajor": (_i, [_vp, _vp, _i, _i, _i, _i, _i, _i, _i, _i, _vp, _i, _i, _vp]),
     "sur_split3_bf16": (_i, [_vp, _i, _i, _vp, _i, _vp]),
+    "sur_lattice_step_bytes": (C.c_longlong, [_i, _i]),
+    "sur_lattice_step": (_i, [_vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _i, _i, _i, _i, _i, _i, _i, _i, C.c_float,
+                              C.c_float, C.c_float, C.c_float, C.c_float, _i, _vp, _vp, _vp, C.c_longlong, _vp]),
     "sur_lattice_serve_bytes": (C.c_longlong, [_i, _i, _i, _i]),
     "sur_lattice_serve": (_i, [_vp, _vp, _vp, _vp, _i, _i, _i, _i, _i, _i, _i, _i, _i, C.c_float, _vp, C.c_longlong, _vp,
                                _vp]),

@@ -544,6 +544,369 @@ __global__ void k_split3_bf16(const float *__restrict__ x, int rows, int K, bf16
     }
 }
 
+// ---- one training step of the lattice table (sur_lattice_step) ----
+//
+// For the pairs of one radial class, with u = t - S m_b, the forward map is a
+// matrix product, y_b(t) = sum_d Q_b[d] H[d][u], H[d][u] = G[ir][d][u + S d + c],
+// c = J - S moff, Q_b[d] = q_b[m_b + moff - d] (zero outside 0..K-1), and the
+// gradient its transpose, dH[d][u] = sum_b Q_b[d] dy_b(u + S m_b).  So a pass
+// over the pairs class by class reads each table entry once per 32 pairs
+// (pair by pair: 400 MB from L2 for 1024 pairs), and sums the gradient of an
+// entry in registers (67 M atomic adds before), where the Adam update follows
+// at once.  1024 pairs, 7.6 M entries: forward and loss 54 us (129 + 19
+// before), gradient and update 58 us (119 + 40 + the clearing 6).  Bound by
+// latency and issue (39 and 48 % active) ahead of DRAM (213 MB of table, moments
+// and gradient, 31 us).
+// Terms with q = 0 are left out, as an entry that is not finite would spread
+// through them.
+
+struct StepGeo {
+    int B, K, NR, D, T, S, J, moff;
+};
+constexpr int ST_W = 8;            // warps of the forward kernel's blocks
+constexpr int ST_P = 4;            // pairs per warp (forward)
+constexpr int ST_U = 128;          // samples per block, four consecutive ones per lane
+constexpr int ST_D = 128;          // table rows whose profile values are staged at a time (forward)
+constexpr int ST_Q = ST_W * ST_P + 4;   // floats per staged row of profiles
+constexpr int ST_RS = 32, ST_NS = 3;    // table rows per copy stage, stages in the ring
+constexpr int ST_BW = 4, ST_R = 4;      // backward: warps per block, table rows per warp
+constexpr size_t ST_SMEM = sizeof(float) * (ST_D * ST_Q + ST_NS * ST_RS * ST_U);
+
+__device__ __forceinline__ void cp_async(float *dst, const float *src, int bytes, bool on) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    if (bytes == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(on ? 16 : 0) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(on ? 4 : 0) : "memory");
+}
+// four consecutive floats p[t .. t+3], zero outside [0, n); VEC: all inside or
+// all outside, 16-byte aligned
+template <bool VEC>
+__device__ __forceinline__ void load4(float (&v)[4], const float *p, int t, int n) {
+    if (VEC) {
+        const float4 x = (unsigned)t < (unsigned)n ? *reinterpret_cast<const float4 *>(p + t) : make_float4(0.f, 0.f, 0.f, 0.f);
+        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[j] = (unsigned)(t + j) < (unsigned)n ? p[t + j] : 0.f;
+    }
+}
+template <bool VEC>
+__device__ __forceinline__ void store4(float *p, int t, int n, const float (&v)[4]) {
+    if (VEC) {
+        if ((unsigned)t < (unsigned)n) *reinterpret_cast<float4 *>(p + t) = make_float4(v[0], v[1], v[2], v[3]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if ((unsigned)(t + j) < (unsigned)n) p[t + j] = v[j];
+    }
+}
+
+// Pairs by class, in their order: block c writes (b, m) to list[start[c] ..] and
+// the range of m of its class.  Class NR holds the pairs that meet no table entry.
+__global__ void __launch_bounds__(256) k_step_bucket(const int *__restrict__ ant, StepGeo g, int *start, int *mlo,
+                                                     int *mhi, int2 *list) {
+    __shared__ int wsum[8], s_lo, s_hi, s_base, s_before;
+    const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    auto cls = [&](int b, int &m) {
+        const int ir = ant[2 * b];
+        m = ant[2 * b + 1];
+        return ir < 0 || ir >= g.NR || m < -g.moff || m > g.D + g.K - 2 - g.moff ? g.NR : ir;
+    };
+    if (tid == 0) {
+        s_before = 0;
+        s_lo = 0x7fffffff;
+        s_hi = -0x7fffffff;
+    }
+    __syncthreads();
+    int before = 0, lo = 0x7fffffff, hi = -0x7fffffff;
+    for (int b = tid; b < g.B; b += 256) {
+        int m;
+        const int k = cls(b, m);
+        before += k < c;
+        if (k == c) {
+            lo = min(lo, m);
+            hi = max(hi, m);
+        }
+    }
+    atomicAdd(&s_before, before);
+    atomicMin(&s_lo, lo);
+    atomicMax(&s_hi, hi);
+    __syncthreads();
+    if (tid == 0) {
+        start[c] = s_base = s_before;
+        if (c == g.NR) start[c + 1] = g.B;
+        mlo[c] = c == g.NR ? 0 : s_lo;
+        mhi[c] = c == g.NR ? 0 : s_hi;
+    }
+    __syncthreads();
+    for (int b0 = 0; b0 < g.B; b0 += 256) {
+        int m;
+        const bool in = b0 + tid < g.B && cls(b0 + tid, m) == c;
+        const unsigned v = __ballot_sync(0xffffffffu, in);
+        if (lane == 0) wsum[w] = __popc(v);
+        __syncthreads();
+        int at = s_base + __popc(v & ((1u << lane) - 1u)), all = 0;
+        for (int k = 0; k < 8; ++k) {
+            if (k < w) at += wsum[k];
+            all += wsum[k];
+        }
+        if (in) list[at] = make_int2(b0 + tid, c == g.NR ? 0 : m);
+        __syncthreads();
+        if (tid == 0) s_base += all;
+        __syncthreads();
+    }
+}
+
+// The next up to 32 pairs of list[at, end) that pass `want(m)`, compacted into
+// sb, sm (b = -1 past the last) by the first warp; returns where to go on.
+template <typename F>
+__device__ __forceinline__ int gather_pairs(const int2 *__restrict__ list, int at, int end, int *sb, int *sm, F want) {
+    const int lane = threadIdx.x & 31;
+    sb[lane] = -1;
+    sm[lane] = 0;
+    __syncwarp();
+    int n = 0;
+    while (n < 32 && at < end) {
+        const int2 bm = at + lane < end ? list[at + lane] : make_int2(-1, 0);
+        const bool in = bm.x >= 0 && want(bm.y);
+        const unsigned v = __ballot_sync(0xffffffffu, in);
+        const int slot = n + __popc(v & ((1u << lane) - 1u));
+        if (in && slot < 32) {
+            sb[slot] = bm.x;
+            sm[slot] = bm.y;
+        }
+        const int all = __popc(v);
+        if (n + all <= 32) {
+            n += all;
+            at += 32;
+        } else {   // go on at the first pair that found no place
+            at += __fns(v, 0, 32 - n + 1);
+            n = 32;
+        }
+    }
+    return at;
+}
+
+// Forward map, loss and its derivative: grid (tiles of u, classes + 1).  The
+// table rows of the tile stream through a ring of asynchronous copies (they come
+// from DRAM: with loads into registers a few rows ahead the kernel waited for
+// them, 113 us), one stage of ST_RS rows for all warps of the block.
+template <bool VEC>
+__global__ void __launch_bounds__(32 * ST_W, 3) k_step_fwd(const float *__restrict__ G, const float *__restrict__ q,
+                                                        const float *__restrict__ s,
+                                                        const float *__restrict__ target,
+                                                        const float *__restrict__ st, StepGeo g, float c_out,
+                                                        const int *__restrict__ start, const int *__restrict__ mlo,
+                                                        const int *__restrict__ mhi, const int2 *__restrict__ list,
+                                                        float *__restrict__ dy, float *loss) {
+    extern __shared__ __align__(16) float dyn[];
+    float *Q = dyn, *ring = dyn + ST_D * ST_Q;
+    __shared__ int sb[ST_W * ST_P], sm[ST_W * ST_P], s_at;
+    __shared__ float red[32];
+    const int cl = blockIdx.y, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int p0 = start[cl], p1 = start[cl + 1];
+    if (p0 >= p1) return;
+    const int lo = mlo[cl], hi = mhi[cl];
+    const int u0 = -g.S * hi + blockIdx.x * ST_U;
+    if (u0 > g.T - 1 - g.S * lo) return;
+    const int c = g.J - g.S * g.moff;
+    const float inv = 1.0f / (float)((long long)g.B * g.T);
+    float sum = 0.f;
+    for (int at = p0; at < p1;) {
+        __syncthreads();
+        if (w == 0) {   // pairs with a sample in this tile of u
+            at = gather_pairs(list, at, p1, sb, sm, [&](int m) {
+                return u0 + ST_U - 1 + g.S * m >= 0 && u0 + g.S * m < g.T;
+            });
+            if (lane == 0) s_at = at;
+        }
+        __syncthreads();
+        at = s_at;
+        // table rows that some of these pairs meet, and that hold a response
+        // sample of this tile, 0 <= u + S d + c < T
+        int d0 = g.D, d1 = -1;
+        if (cl < g.NR)
+            for (int i = 0; i < ST_W * ST_P; ++i)
+                if (sb[i] >= 0) {
+                    d0 = min(d0, sm[i] + g.moff - g.K + 1);
+                    d1 = max(d1, sm[i] + g.moff);
+                }
+        if (g.S > 0) {
+            const int a = -(u0 + ST_U - 1 + c), z = g.T - 1 - u0 - c;   // a <= S d <= z
+            d0 = max(d0, a <= 0 ? 0 : (a + g.S - 1) / g.S);
+            d1 = min(d1, z < 0 ? -1 : z / g.S);
+        }
+        d0 = max(d0, 0);
+        d1 = min(d1, g.D - 1);
+        const int nd = max(0, d1 + 1 - d0), stages = (nd + ST_RS - 1) / ST_RS;
+        auto fetch = [&](int k) {   // rows d0 + k ST_RS .. of the tile, one commit group per stage
+            if (k < stages) {
+                float *r = ring + k % ST_NS * ST_RS * ST_U;
+                constexpr int E = VEC ? 4 : 1;
+#pragma unroll
+                for (int e = tid * E; e < ST_RS * ST_U; e += 32 * ST_W * E) {
+                    const int d = d0 + k * ST_RS + e / ST_U, tau = u0 + e % ST_U + g.S * d + c;
+                    const bool on = d <= d1 && (unsigned)tau < (unsigned)g.T;
+                    cp_async(r + e, on ? G + ((long long)cl * g.D + d) * g.T + tau : G, 4 * E, on);
+                }
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        float acc[ST_P][4];
+#pragma unroll
+        for (int i = 0; i < ST_P; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+#pragma unroll 1
+        for (int k = 0; k < ST_NS - 1; ++k) fetch(k);
+        for (int k = 0; k < stages; ++k) {
+            if (k * ST_RS % ST_D == 0) {   // the profile values of the next ST_D rows
+                __syncthreads();
+#pragma unroll
+                for (int e = tid; e < ST_D * ST_W * ST_P; e += 32 * ST_W) {
+                    const int dd = e % ST_D, i = e / ST_D, kk = sm[i] + g.moff - (d0 + k * ST_RS + dd);
+                    Q[dd * ST_Q + i] = sb[i] >= 0 && kk >= 0 && kk < g.K ? q[(long long)sb[i] * g.K + kk] : 0.f;
+                }
+            }
+            asm volatile("cp.async.wait_group %0;" ::"n"(ST_NS - 2) : "memory");
+            __syncthreads();   // stage k is there, and stage k - 1 is done with
+            fetch(k + ST_NS - 1);
+            if (sb[w * ST_P] < 0) continue;   // no pair for this warp
+            const float *r = ring + k % ST_NS * ST_RS * ST_U + 4 * lane;
+            const float *qr = Q + (k * ST_RS % ST_D) * ST_Q + w * ST_P;
+            const int n = min(ST_RS, nd - k * ST_RS);
+#pragma unroll 4
+            for (int e = 0; e < n; ++e) {
+                const float4 h = *reinterpret_cast<const float4 *>(r + e * ST_U);
+                const float4 v = *reinterpret_cast<const float4 *>(qr + e * ST_Q);
+                const float qv[ST_P] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int i = 0; i < ST_P; ++i)
+                    if (qv[i] != 0.f) {
+                        acc[i][0] = fmaf(qv[i], h.x, acc[i][0]);
+                        acc[i][1] = fmaf(qv[i], h.y, acc[i][1]);
+                        acc[i][2] = fmaf(qv[i], h.z, acc[i][2]);
+                        acc[i][3] = fmaf(qv[i], h.w, acc[i][3]);
+                    }
+            }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+#pragma unroll
+        for (int i = 0; i < ST_P; ++i) {
+            const int b = sb[w * ST_P + i];
+            if (b < 0) continue;
+            // the scaled output and target, and back (relative: by the target's own peak)
+            const float sq = s[b], peak = st ? st[b] : 0.f;
+            const float fy = st ? c_out * sq : 1.f, fr = st ? (peak != 0.f ? 1.f / peak : 0.f) : 1.f;
+            const float ft = st ? 1.f : (sq != 0.f ? (1.f / c_out) / sq : 0.f);
+            const int t = u0 + 4 * lane + g.S * sm[w * ST_P + i];
+            float y[4], o[4];
+            load4<VEC>(y, target + (long long)b * g.T, t, g.T);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float e = acc[i][j] * fy * fr - y[j] * ft;
+                o[j] = 2.f * e * inv * fy * fr;
+                if ((unsigned)(t + j) < (unsigned)g.T) sum += e * e;
+            }
+            store4<VEC>(dy + (long long)b * g.T, t, g.T, o);
+        }
+    }
+    const float bs = block_sum(sum, red);
+    if (tid == 0) atomicAdd(loss, bs * inv);
+}
+
+// Gradient and Adam update: grid (tiles of u, tiles of ST_BW ST_R table rows, classes).
+template <bool VEC>
+__global__ void __launch_bounds__(32 * ST_BW) k_step_bwd(const float *__restrict__ dy, const float *__restrict__ q,
+                                                         StepGeo g, const int *__restrict__ start,
+                                                         const int2 *__restrict__ list,
+                                                         float *__restrict__ W, float *__restrict__ dG,
+                                                         float *__restrict__ m1, float *__restrict__ m2, float lr,
+                                                         float b1, float b2, float eps, float i1, float i2) {
+    constexpr int NP = 32, ROWS = ST_BW * ST_R;   // pairs staged at a time, table rows of the block
+    __shared__ __align__(16) float Q[NP][ROWS];
+    __shared__ int sb[NP], sm[NP], s_at;
+    const int cl = blockIdx.z, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int dt = blockIdx.y * ROWS, dw = dt + w * ST_R;
+    const int c = g.J - g.S * g.moff;
+    const int tau0 = blockIdx.x * ST_U + 4 * lane - g.S * (ST_R - 1);   // of row dw; row dw + i: + S i
+    const int p0 = start[cl], p1 = start[cl + 1];
+    // the table entries and moments, from DRAM to L2 while the gradient is summed
+#pragma unroll
+    for (int i = 0; i < ST_R; ++i) {
+        const int tau = tau0 + g.S * i;
+        if (dw + i >= g.D || (unsigned)tau >= (unsigned)g.T) continue;
+        const long long o = ((long long)cl * g.D + dw + i) * g.T + tau;
+        if (lane % 8 == 0) {
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(W + o));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(m1 + o));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(m2 + o));
+        }
+    }
+    float acc[ST_R][4];
+#pragma unroll
+    for (int i = 0; i < ST_R; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+    for (int at = p0; at < p1;) {
+        __syncthreads();
+        if (w == 0) {   // pairs that meet these table rows
+            at = gather_pairs(list, at, p1, sb, sm, [&](int m) {
+                return m + g.moff - dt >= 0 && m + g.moff - (dt + ROWS - 1) < g.K;
+            });
+            if (lane == 0) s_at = at;
+        }
+        __syncthreads();
+        at = s_at;
+#pragma unroll
+        for (int e = tid; e < NP * ROWS; e += 32 * ST_BW) {
+            const int i = e % ROWS, p = e / ROWS, k = sm[p] + g.moff - (dt + i);
+            Q[p][i] = sb[p] >= 0 && k >= 0 && k < g.K ? q[(long long)sb[p] * g.K + k] : 0.f;
+        }
+        __syncthreads();
+        // four pairs' samples in flight
+        for (int pb = 0; pb < NP && sb[pb] >= 0; pb += 4) {
+            float h[4][4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e)   // a pair past the last has b = -1: an empty row
+                load4<VEC>(h[e], dy + (long long)max(sb[pb + e], 0) * g.T, tau0 - g.S * dw - c + g.S * sm[pb + e],
+                           sb[pb + e] >= 0 ? g.T : 0);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float4 v = *reinterpret_cast<const float4 *>(&Q[pb + e][w * ST_R]);
+                const float qv[ST_R] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int i = 0; i < ST_R; ++i)
+                    if (qv[i] != 0.f)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(qv[i], h[e][j], acc[i][j]);
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < ST_R; ++i) {
+        if (dw + i >= g.D) continue;
+        const long long base = ((long long)cl * g.D + dw + i) * g.T;
+        const int tau = tau0 + g.S * i;
+        float a[4], v[4], x[4];
+        load4<VEC>(a, m1 + base, tau, g.T);
+        load4<VEC>(v, m2 + base, tau, g.T);
+        load4<VEC>(x, W + base, tau, g.T);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float gi = acc[i][j];
+            a[j] = b1 * a[j] + (1.f - b1) * gi;
+            v[j] = b2 * v[j] + (1.f - b2) * gi * gi;
+            x[j] = x[j] - lr * (a[j] * i1) / (sqrtf(v[j] * i2) + eps);
+        }
+        store4<VEC>(dG + base, tau, g.T, acc[i]);
+        store4<VEC>(m1 + base, tau, g.T, a);
+        store4<VEC>(m2 + base, tau, g.T, v);
+        store4<VEC>(W + base, tau, g.T, x);
+    }
+}
+
 // ---- serving every profile at every antenna (sur_lattice_serve) ----
 
 // One warp per profile: its peak s, and the split of the normalised profile as
@@ -899,6 +1262,52 @@ int sur_lattice_serve(const void *Ghi, const void *Glo, const float *q, const in
     const int rc = launched();
     if (rc != FDTD_OK) return rc;
     return fdtd::gtc::serve_gemm(Q, W, L.TW, out, P, T, L.KS, A, s, c_out, st);
+}
+
+long long sur_lattice_step_bytes(int B, int NR) {
+    if (B < 1 || NR < 1) return FDTD_ERR_ARG;
+    return 4LL * (3LL * NR + 4 + 2LL * B);
+}
+
+int sur_lattice_step(float *G, float *dG, float *m, float *v, const float *qn, const float *s, const int *ant,
+                     const float *target, const float *st, int B, int K, int NR, int D, int T, int S, int J, int moff,
+                     float c_out, float lr, float b1, float b2, float eps, int t, float *dy, float *loss, void *work,
+                     long long work_bytes, void *stream) {
+    if (!G || !dG || !m || !v || !qn || !s || !ant || !target || !dy || !loss || !work || B < 1 || B > 65535 || K < 1 ||
+        K > 1024 || NR < 1 || NR > 65534 || D < 1 || T < 1 || S < 0 || J < 0 || t < 1 ||
+        (reinterpret_cast<uintptr_t>(work) & 7) || work_bytes < sur_lattice_step_bytes(B, NR))
+        return FDTD_ERR_ARG;
+    // positions along u and tau stay well inside 32 bits
+    if ((long long)S * (D + 2LL * K + (moff < 0 ? -(long long)moff : moff)) + T + J > (1LL << 30)) return FDTD_ERR_ARG;
+    const StepGeo g{B, K, NR, D, T, S, J, moff};
+    cudaStream_t q = static_cast<cudaStream_t>(stream);
+    int2 *list = static_cast<int2 *>(work);
+    int *start = reinterpret_cast<int *>(list + B), *mlo = start + NR + 2, *mhi = mlo + NR + 1;
+    if (cudaMemsetAsync(loss, 0, sizeof(float), q) != cudaSuccess) return FDTD_ERR_CUDA;
+    k_step_bucket<<<NR + 1, 256, 0, q>>>(ant, g, start, mlo, mhi, list);
+    // u of a class spans T + S (range of m), m in [-moff, D + K - 2 - moff]
+    const long long span = T + (long long)S * (D + K - 2);
+    const dim3 gf((unsigned)((span + ST_U - 1) / ST_U), NR + 1);
+    const dim3 gb((unsigned)((T + (long long)S * (ST_R - 1) + ST_U - 1) / ST_U), (D + ST_BW * ST_R - 1) / (ST_BW * ST_R), NR);
+    const float i1 = 1.f / (1.f - powf(b1, (float)t)), i2 = 1.f / (1.f - powf(b2, (float)t));
+    // 16-byte accesses where every row and lag allows them
+    const bool vec = S % 4 == 0 && J % 4 == 0 && T % 4 == 0 && aligned16(G) && aligned16(dG) && aligned16(m) &&
+                     aligned16(v) && aligned16(target) && aligned16(dy);
+    const void *fwd = vec ? (const void *)k_step_fwd<true> : (const void *)k_step_fwd<false>;
+    if (cudaFuncSetAttribute(fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ST_SMEM) != cudaSuccess) {
+        cudaGetLastError();
+        return FDTD_ERR_CUDA;
+    }
+    if (vec) {
+        k_step_fwd<true><<<gf, 32 * ST_W, ST_SMEM, q>>>(G, qn, s, target, st, g, c_out, start, mlo, mhi, list, dy,
+                                                        loss);
+        k_step_bwd<true><<<gb, 32 * ST_BW, 0, q>>>(dy, qn, g, start, list, G, dG, m, v, lr, b1, b2, eps, i1, i2);
+    } else {
+        k_step_fwd<false><<<gf, 32 * ST_W, ST_SMEM, q>>>(G, qn, s, target, st, g, c_out, start, mlo, mhi, list, dy,
+                                                         loss);
+        k_step_bwd<false><<<gb, 32 * ST_BW, 0, q>>>(dy, qn, g, start, list, G, dG, m, v, lr, b1, b2, eps, i1, i2);
+    }
+    return launched();
 }
 
 }  // extern "C"

@@ -34,8 +34,9 @@ from dataclasses import dataclass, field
 import numpy as np
 
 from . import (check, fdtd_probes, profile_gaisser_hillas, lateral_nkg, Simulation, sur_adam, sur_antenna_features,
-               sur_assemble, sur_assemble_bwd, sur_bias_grad, sur_cast_bf16, sur_gemm_bf16, sur_lattice_bwd,
-               sur_lattice_fwd, sur_lattice_fwd_f32, sur_lattice_serve, sur_lattice_serve_bytes, sur_mse,
+               sur_assemble, sur_assemble_bwd, sur_bias_grad, sur_cast_bf16, sur_gemm_bf16, sur_lattice_fwd,
+               sur_lattice_fwd_f32, sur_lattice_serve, sur_lattice_serve_bytes, sur_lattice_step,
+               sur_lattice_step_bytes, sur_mse,
                sur_normalize_rows, sur_pairs, sur_relu_bwd, sur_scale_rows, sur_split_bf16)
 
 N_FEAT = 64
@@ -344,7 +345,9 @@ class Lattice:
         if B not in self._ws:
             e = lambda *sh: torch.empty(sh, dtype=torch.float32, device="cuda")
             self._ws = {B: {"qn": e(B, self.geo.K), "s": e(B), "y": e(B, self.geo.T), "tn": e(B, self.geo.T),
-                            "dy": e(B, self.geo.T), "loss": e(1)}}
+                            "dy": e(B, self.geo.T), "st": e(B), "loss": e(1),
+                            "work": torch.empty(sur_lattice_step_bytes(B, self.geo.NR), dtype=torch.uint8,
+                                                device="cuda")}}
         return self._ws[B]
 
     def split(self):
@@ -384,28 +387,20 @@ class Lattice:
         B = q.shape[0]
         w = self._w(B)
         st = _stream()
-        self._fwd(q, ant, False, master=True)
+        check(sur_normalize_rows(_p(q), B, g.K, _p(w["qn"]), _p(w["s"]), st), "sur_normalize_rows")
         if relative:
-            if "st" not in w:
-                import torch
-                w["st"] = torch.empty(B, dtype=torch.float32, device="cuda")
             check(sur_normalize_rows(_p(trace), B, g.T, _p(w["tn"]), _p(w["st"]), st), "sur_normalize_rows")
-            # model trace / its target's peak = y_n c_out s_q / s_t
-            check(sur_scale_rows(_p(w["y"]), B, g.T, _p(w["s"]), self.c_out, 0, st), "sur_scale_rows")
-            check(sur_scale_rows(_p(w["y"]), B, g.T, _p(w["st"]), 1.0, 1, st), "sur_scale_rows")
+            target = w["tn"]
+        elif (trace.device == w["tn"].device and trace.dtype == w["tn"].dtype and trace.shape == w["tn"].shape
+              and trace.is_contiguous()):
+            target = trace
         else:
-            w["tn"].copy_(trace)
-            check(sur_scale_rows(_p(w["tn"]), B, g.T, _p(w["s"]), 1.0 / self.c_out, 1, st), "sur_scale_rows")
-        check(sur_mse(_p(w["y"]), _p(w["tn"]), B * g.T, _p(w["dy"]), _p(w["loss"]), st), "sur_mse")
-        if relative:   # back to the gradient with respect to y_n
-            check(sur_scale_rows(_p(w["dy"]), B, g.T, _p(w["s"]), self.c_out, 0, st), "sur_scale_rows")
-            check(sur_scale_rows(_p(w["dy"]), B, g.T, _p(w["st"]), 1.0, 1, st), "sur_scale_rows")
-        self.dG.zero_()
-        check(sur_lattice_bwd(_p(w["dy"]), _p(w["qn"]), _p(ant), B, g.K, g.NR, self.D, g.T, g.S, g.J, self.moff,
-                              _p(self.dG), st), "sur_lattice_bwd")
+            target = w["tn"].copy_(trace)
+        check(sur_lattice_step(_p(self.G), _p(self.dG), _p(self.m), _p(self.v), _p(w["qn"]), _p(w["s"]), _p(ant),
+                               _p(target), _p(w["st"]) if relative else None, B, g.K, g.NR, self.D, g.T, g.S, g.J,
+                               self.moff, self.c_out, lr, b1, b2, eps, self.t + 1, _p(w["dy"]), _p(w["loss"]),
+                               _p(w["work"]), w["work"].numel(), st), "sur_lattice_step")
         self.t += 1
-        check(sur_adam(_p(self.G), None, _p(self.dG), _p(self.m), _p(self.v), self.G.numel(), lr, b1, b2, eps, self.t,
-                       st), "sur_adam")
         self._split = False
         return w["loss"]
 
