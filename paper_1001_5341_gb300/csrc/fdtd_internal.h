@@ -150,6 +150,7 @@ struct fdtd_ctx {
                               // 2 two steps per pass (vector tile for a last odd step)
     void *vtile;              // host state of the vector-tile path
     void *tb2;                // host state of the two-step path
+    void *res;                // host state of the resident path (null: not for this grid)
     int *d_flags;             // device error flags (bits 0-1: a bounded wait gave up,
                               // bit 2: the watchdog saw a non-finite value)
     int watch_every;          // steps between watchdog checks (0: off)
@@ -219,6 +220,17 @@ void launch_tb2_probes(fdtd_ctx *h, cudaStream_t s);   // detector slots n, n+1 
 const char *tb2_name(const fdtd_ctx *h);
 void tb2_release(fdtd_ctx *h);
 float *tb2_probe_values(fdtd_ctx *h);   // the pass's records of E^{n+1} (6 per detector)
+
+// Many steps of a small PEC or Mur grid in one launch, fields resident on chip
+// (kernels_res.cu); taken in the place of the one-step path where res_ready
+void res_prepare(fdtd_ctx *h);
+void res_release(fdtd_ctx *h);
+void res_set_probes(fdtd_ctx *h);                    // after the detectors changed
+bool res_ready(fdtd_ctx *h, cudaStream_t s);
+int res_steps();                                     // most steps per launch
+bool launch_res(fdtd_ctx *h, int n, cudaStream_t s); // advances h->cur and h->steps
+// detector slots steps .. steps + n - 1 from records [n][np][6] of E (kernels_basic.cu)
+void launch_record_probes(const fdtd_ctx *h, cudaStream_t s, const float *rec, int n);
 
 // host tables (tables.cpp)
 void cpml_coefficients(int n, int P, double dx, double dt, double eps_r, float *aE, float *bE,

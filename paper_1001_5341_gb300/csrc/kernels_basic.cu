@@ -113,6 +113,20 @@ __global__ void k_probes2(Grid g, const float *__restrict__ E, Probes p, long lo
     readout_fields(g, E, p, t, slot + 1);
 }
 
+// n steps' detectors from the resident path's records: step blockIdx.y.
+__global__ void k_record_probes(Probes p, long long slot, const float *__restrict__ rec) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= p.n) return;
+    float v[6];
+    for (int s = 0; s < 6; ++s) v[s] = rec[6 * ((long long)blockIdx.y * p.n + t) + s];
+    readout(p, t, slot + blockIdx.y, v);
+}
+
+void launch_record_probes(const fdtd_ctx *h, cudaStream_t s, const float *rec, int n) {
+    Probes p{h->np, h->max_steps, h->d_ijk, h->d_cxy, h->d_trace};
+    k_record_probes<<<dim3((h->np + 127) / 128, n), 128, 0, s>>>(p, h->steps, rec);
+}
+
 void launch_probes(const fdtd_ctx *h, cudaStream_t s) {
     Probes p{h->np, h->max_steps, h->d_ijk, h->d_cxy, h->d_trace};
     k_probes<<<(h->np + 127) / 128, 128, 0, s>>>(h->g, h->fields[h->cur ^ 1], p, h->steps);
