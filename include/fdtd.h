@@ -226,12 +226,12 @@ const char *fdtd_kernel_name(fdtd_t h);
  *       recomputes the first step on a two-cell halo, so a pass reads the
  *       fields once and writes them once for two steps; CPML and detectors
  *       included; a last odd step of fdtd_step runs on path 1.  PEC and CPML
- *       grids only (FDTD_ERR_ARG on a Mur grid); the default there from
- *       FDTD_TWO_STEP_MIN_CELLS cells, about 12.6 million (on smaller grids
- *       its blocks are too few to hide their start-up: measured 22 against
- *       28 Gcell/s for path 1 on 96 x 96 x 384, CPML 10, and 52.5 against
- *       50.7 on 128 x 128 x 512, where path 1 is faster with thousands of
- *       detectors in one tile; 69.5 against 52.2 on 160 x 160 x 640);
+ *       grids only (FDTD_ERR_ARG on a Mur grid).  The default of PEC grids
+ *       that do not fit the resident runs of path 1 (100^3: 20.7 -> 18.6 us a
+ *       step), of CPML grids of up to 128 columns from 2.5 million cells
+ *       (128 x 128 x 512, CPML 10: 124 -> 93; 128^3: 49 against 52) and of
+ *       other CPML grids from FDTD_TWO_STEP_MIN_CELLS cells, about 12.6 million
+ *       (160 x 160 x 640: 274 -> 174; 200^3: 116 against 117.5);
  *   1 = one pass per step: TMA-staged vector-tile z-march over the whole
  *       grid, CPML included (the default on Mur grids and smaller grids).
  *       Runs of two steps or more of a small PEC or Mur grid (nx <= 127, and

@@ -60,6 +60,16 @@ void release(fdtd_ctx *h) {
     delete h;
 }
 
+// Fewest cells for which the two-step path is the default.  Measured, us a step,
+// path 1 and path 2: PEC grids too large for the resident path 20.7, 18.6 (100^3),
+// 31.5, 21.6 (150x100x100), 87.6, 44 (128x128x512); CPML grids of one tile column
+// 49.4, 51.9 (128^3), 68.0, 52.2 (128x128x160), 48.6 against 73.9 on 64x64x400 but
+// 49.1 against 45.3 on 96x96x160; other CPML grids 61.8, 67.0 (200x200x80), 115.8,
+// 117.5 (200^3), 140.4, 110.4 (300x200x150), 171.8, 158.2 (200x200x300).
+long long two_step_min_cells(const fdtd_ctx *h) {
+    return h->P == 0 ? 0 : h->g.nx <= 128 ? 2500000 : FDTD_TWO_STEP_MIN_CELLS;
+}
+
 int interior_lo(const fdtd_ctx *h) { return h->boundary == FDTD_CPML ? h->P + 1 : 1; }
 
 size_t field_bytes(const fdtd_ctx *h) { return sizeof(float) * 6 * (size_t)h->g.comp; }
@@ -128,7 +138,7 @@ int fdtd_step_on(fdtd_ctx *h, int n, cudaStream_t st) {
             }
             res_release(h);   // refused: the one-step path from here on
         }
-        if (h->kernel == 2 && n - s >= 2) {
+        if (h->kernel == 2 && n - s >= 2 && tb2_ready(h)) {
             // two steps in one pass; the detectors of both from its records
             timed_launch(h, st, [](const fdtd_ctx *c, cudaStream_t q) { launch_tb2(const_cast<fdtd_ctx *>(c), q); });
             if (h->np > 0) { launch_tb2_probes(h, st); h->launches++; }
@@ -282,7 +292,7 @@ int fdtd_create(fdtd_t *out, int nx, int ny, int nz, double dx, double dt, doubl
         h->kernel = 1;
         res_prepare(h);
     }
-    if ((long long)nx * ny * nz >= FDTD_TWO_STEP_MIN_CELLS && tb2_prepare(h) == FDTD_OK) h->kernel = 2;
+    if (!h->res && (long long)nx * ny * nz >= two_step_min_cells(h) && tb2_prepare(h) == FDTD_OK) h->kernel = 2;
     cudaGetLastError();
     *out = h;
     return FDTD_OK;

@@ -219,7 +219,9 @@ void launch_tb2(fdtd_ctx *h, cudaStream_t s);          // steps n, n+1
 void launch_tb2_probes(fdtd_ctx *h, cudaStream_t s);   // detector slots n, n+1 after launch_tb2
 const char *tb2_name(const fdtd_ctx *h);
 void tb2_release(fdtd_ctx *h);
-float *tb2_probe_values(fdtd_ctx *h);   // the pass's records of E^{n+1} (6 per detector)
+// the pass's E^{n+1} for the detectors, and the places of the six values of each
+const float *tb2_probe_values(const fdtd_ctx *h, const int **pos);
+bool tb2_ready(fdtd_ctx *h);
 
 // Many steps of a small PEC or Mur grid in one launch, fields resident on chip
 // (kernels_res.cu); taken in the place of the one-step path where res_ready

@@ -101,14 +101,14 @@ __global__ void k_probes(Grid g, const float *__restrict__ E, Probes p, long lon
     readout_fields(g, E, p, t, slot);
 }
 
-// After a two-step pass: slot n from the pass's records of E^{n+1} (six
-// values per detector), slot n+1 from E^{n+2} (set cur^1).
+// After a two-step pass: slot n from the rows of E^{n+1} that the pass stored
+// (pos: the places of the six values per detector), slot n+1 from E^{n+2} (set cur^1).
 __global__ void k_probes2(Grid g, const float *__restrict__ E, Probes p, long long slot,
-                          const float *__restrict__ rec) {
+                          const float *__restrict__ rec, const int *__restrict__ pos) {
     int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= p.n) return;
     float v[6];
-    for (int s = 0; s < 6; ++s) v[s] = rec[6 * t + s];
+    for (int s = 0; s < 6; ++s) v[s] = rec[pos[6 * t + s]];
     readout(p, t, slot, v);
     readout_fields(g, E, p, t, slot + 1);
 }
@@ -134,9 +134,10 @@ void launch_probes(const fdtd_ctx *h, cudaStream_t s) {
 
 void launch_tb2_probes(fdtd_ctx *h, cudaStream_t s) {
     Probes p{h->np, h->max_steps, h->d_ijk, h->d_cxy, h->d_trace};
-    const float *rec = tb2_probe_values(h);
+    const int *pos = nullptr;
+    const float *rec = tb2_probe_values(h, &pos);
     if (!rec) return;
-    k_probes2<<<(h->np + 127) / 128, 128, 0, s>>>(h->g, h->fields[h->cur ^ 1], p, h->steps, rec);
+    k_probes2<<<(h->np + 127) / 128, 128, 0, s>>>(h->g, h->fields[h->cur ^ 1], p, h->steps, rec, pos);
 }
 
 // Watchdog of the step path: block (x, y) scans plane k = min(y * stride,

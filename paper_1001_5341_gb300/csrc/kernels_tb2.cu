@@ -7,6 +7,11 @@
 // the fields are read once and written once for two steps, 24 B + 24 B per
 // cell, so 24 B per cell-update instead of 48 B.
 //
+// A grid of up to 128 columns is one wide tile of all its columns, x layers
+// included (nothing lies beyond its ends, so it needs no halo there): with a wide
+// tile between two narrow ones 128x128x512 (10 CPML cells) took 144 us a step,
+// with one full tile 106 (93 with the chunks of launch_time); PEC 90 -> 46.
+//
 // Tiles.  A wide block owns up to 120 columns [i0, i0+120) by TY = 8 rows
 // [j0, j0+8) and marches up a chunk of z planes [k0, k1).  It computes the
 // first step (level 1: H^{n+1/2}, E^{n+1}) on a larger region and the second
@@ -69,10 +74,8 @@
 // Detectors.  The level-1 E of the six cells of a detector's readout (Ex at
 // i-1, i; Ey at j-1, j; Ez at k-1, k) go to a small buffer from the tile that
 // owns them; the readout of step n+1 reads them, that of step n+2 reads the
-// fields.  A block's records are sorted by plane; those of plane q are served
-// in the next iteration, one per thread, from the shared rows that hold the
-// level-1 E of plane q (Ex, Ez in the exchange rows, Ey in rows of its own),
-// so thousands of detectors in one tile cost a few loads per plane.
+// fields.  Each owned row of a block has the list of planes that some readout
+// takes a value from; the row's warp stores its level-1 E of those planes.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -92,8 +95,10 @@ using namespace tma;
 constexpr int TY = 8;                 // owned rows
 constexpr int NWR = TY + 3;           // row warps: rows j0-2 .. j0+TY
 constexpr int NT = 32 * (NWR + 1);    // and one warp that refills the stage ring
-constexpr int BR = TY + 4;            // box rows j0-2 .. j0+TY+1
+constexpr int BR = TY + 4;            // rows j0-2 .. j0+TY+1 (Ex and Ez boxes, coefficient table)
+constexpr int PR = NWR;               // rows of the other field boxes and the psi boxes
 constexpr int NSMAX = 8;
+constexpr int PROW = 3 * 128;         // floats of a stored row of level-1 E (a wide tile's)
 
 // mbarriers of a block: the stage ring (full: the stage's copies landed;
 // empty: every row warp is done with it) and the exchange rows (a row warp's
@@ -111,11 +116,19 @@ template <int VW>
 struct Geo {
     static constexpr int TXC = 32 * VW;          // computed columns i0-4 .. i0+TXC-5
     static constexpr int TXO = TXC - 8;          // owned columns (lanes 4/VW .. 31-4/VW)
-    static constexpr int BOX = TXC * BR;         // floats of a field or y/z psi box
-    static constexpr int FIELDS = 6 * BOX;
+    static constexpr int PBOX = TXC * PR;        // floats of a y/z psi box
+    // field boxes of a stage, component c (Ex Ey Ez Hx Hy Hz): rows, offset
+    __host__ __device__ static constexpr int frows(int c) { return c == 0 || c == 2 ? BR : PR; }
+    __host__ __device__ static constexpr int foff(int c) {
+        return TXC * (c * PR + (c > 0 ? BR - PR : 0) + (c > 2 ? BR - PR : 0));
+    }
+    static constexpr int FIELDS = foff(6);
     static constexpr unsigned FIELD_BYTES = 4u * FIELDS;
     static constexpr int XROW = 2 * TXC;         // exchange floats per warp row (two components)
-    static constexpr int XBUF = NWR * XROW;      // one exchange buffer
+    // exchange buffers: A's two (rows w = 0 .. 9 are read), B's (2 .. 10; row 1
+    // is written), C's (1 .. 8; row 9 is written)
+    static constexpr int XA_ROWS = NWR - 1, XB_ROWS = NWR - 1, XC_ROWS = NWR - 2;
+    static constexpr int XFLOATS = (2 * XA_ROWS + XB_ROWS + XC_ROWS) * XROW;
     // CPML coefficient table (floats): aH, bH, aE, bE of the computed columns,
     // of the rows j0-2 .. j0+TY+1, of the planes kstart .. kstart+zt-1
     static constexpr int CX = 0;
@@ -126,7 +139,7 @@ struct Geo {
     // shared memory: barriers, four exchange buffers (A's two, B's, C's),
     // coefficient table, ring
     __host__ __device__ static constexpr int head_floats(int zt) {
-        return (4 * XBUF + CZ + 4 * zt + 31) / 32 * 32;
+        return (XFLOATS + CZ + 4 * zt + 31) / 32 * 32;
     }
 };
 
@@ -209,13 +222,18 @@ struct Maps {
 // [0, a), nw wide ones (float4 lanes, up to 120) over [a, b), then narrow ones
 // over [b, nx).  On a CPML grid the wide tiles stay clear of the x layers
 // (their owned results depend on columns i0-2 .. end+1 only), so the x layers'
-// CPML memory is updated by the narrow tiles alone, one column per lane.
+// CPML memory is updated by the narrow tiles alone, one column per lane.  A
+// grid of up to 128 columns is one wide tile of all columns (full).
 struct TileCol {
     int i0, w, vw;
 };
-__host__ __device__ inline TileCol tile_col(int tc, int a, int b, int nl, int nw, int nx) {
+__host__ __device__ inline TileCol tile_col(int tc, int a, int b, int nl, int nw, int nx, bool full) {
     TileCol t;
-    if (tc < nl) {
+    if (full) {
+        t.i0 = 4;   // computed columns 0 .. 127
+        t.w = nx - 4;
+        t.vw = 4;
+    } else if (tc < nl) {
         t.i0 = 24 * tc;
         t.w = a - t.i0 < 24 ? a - t.i0 : 24;
         t.vw = 1;
@@ -247,9 +265,9 @@ struct Args {
     SourceStep ss1, ss2;    // current of steps n and n+1
     float kE, kH;
     int *flags;
-    const int4 *prec;       // detector records {k, j, i, slot * 4 + component}
-    const int *pidx;        // records of block b: [pidx[b], pidx[b+1])
-    float *pbuf;            // level-1 values of the records
+    const int *planes;      // planes whose level-1 E detectors read, in lists
+    const int *pidx;        // list of owned row t of block b: [pidx[b TY + t], pidx[b TY + t + 1])
+    float *pbuf;            // [plane in a list][PROW]: level-1 Ex, Ey, Ez of the tile's columns
 };
 
 struct Blk {
@@ -259,7 +277,7 @@ struct Blk {
     int l0;                 // first y slab row of the y box
     int xo, yo, zo, stage, ns;
     int xlo, xhi, nxb, xb;
-    int pbeg, pend;
+    int rec;                // first of the block's TY record lists
 };
 
 template <int VW>
@@ -269,13 +287,13 @@ __device__ __forceinline__ void issue_plane(const Args &A, const Maps &M, const 
     const int p = B.kstart + r;
     const int lz = (B.hz && p >= 0 && p < A.g.nz) ? slab_cell(p, A.g.nz, A.pm.P) : -1;
     unsigned bytes = G::FIELD_BYTES;
-    if (B.hx) bytes += 16u * (unsigned)(B.nxb * A.xbw * BR);
-    if (B.hy) bytes += 16u * G::BOX;
-    if (lz >= 0) bytes += 16u * G::BOX;
+    if (B.hx) bytes += 16u * (unsigned)(B.nxb * A.xbw * PR);
+    if (B.hy) bytes += 16u * G::PBOX;
+    if (lz >= 0) bytes += 16u * G::PBOX;
     mbar_expect_tx(bar, bytes);
     constexpr int WD = VW == 4 ? 0 : 1;
 #pragma unroll
-    for (int c = 0; c < 6; ++c) tma_load(st + c * G::BOX, &M.f[WD][A.cur][c], bar, B.i0 - 4, B.j0 - 2, p);
+    for (int c = 0; c < 6; ++c) tma_load(st + G::foff(c), &M.f[WD][A.cur][c], bar, B.i0 - 4, B.j0 - 2, p);
     if (B.hx)
         for (int a = 0; a < 4; ++a) {
             float *d = st + B.xo + a * B.nxb * B.xb;
@@ -285,10 +303,10 @@ __device__ __forceinline__ void issue_plane(const Args &A, const Maps &M, const 
         }
     if (B.hy)
         for (int a = 0; a < 4; ++a)
-            tma_load(st + B.yo + a * G::BOX, &M.y[WD][a][a < 2 ? A.cur : A.ecur], bar, B.i0 - 4, B.l0, p);
+            tma_load(st + B.yo + a * G::PBOX, &M.y[WD][a][a < 2 ? A.cur : A.ecur], bar, B.i0 - 4, B.l0, p);
     if (lz >= 0)
         for (int a = 0; a < 4; ++a)
-            tma_load(st + B.zo + a * G::BOX, &M.z[WD][a][a < 2 ? A.cur : A.ecur], bar, B.i0 - 4, B.j0 - 2, lz);
+            tma_load(st + B.zo + a * G::PBOX, &M.z[WD][a][a < 2 ? A.cur : A.ecur], bar, B.i0 - 4, B.j0 - 2, lz);
 }
 
 template <int VW>
@@ -330,6 +348,20 @@ __device__ __forceinline__ Masks<typename Vec<VW>::U> masks(const Lane<VW> &L, i
 
 constexpr unsigned FULL = 0xffffffffu;
 
+// The neighbour lane's value across the end of the vector.  Beyond lanes 0 and
+// 31 a full tile reads the zeros outside the grid; in the other tiles that value
+// reaches no owned cell.
+template <bool FT>
+__device__ __forceinline__ float from_right(float v, int lane) {
+    const float r = __shfl_down_sync(FULL, v, 1);
+    return FT && lane == 31 ? 0.f : r;
+}
+template <bool FT>
+__device__ __forceinline__ float from_left(float v, int lane) {
+    const float l = __shfl_up_sync(FULL, v, 1);
+    return FT && lane == 0 ? 0.f : l;
+}
+
 // Register state carried from one iteration to the next.
 template <typename V>
 struct State {
@@ -345,42 +377,18 @@ struct RingPos {
     uint32_t ph1;
 };
 
-// element e of lane src's vector (every lane of the warp takes part)
-__device__ __forceinline__ float shfl_elem(float v, int src, int) { return __shfl_sync(0xffffffffu, v, src); }
-__device__ __forceinline__ float shfl_elem(float4 v, int src, int e) {
-    const float x = __shfl_sync(0xffffffffu, v.x, src), y = __shfl_sync(0xffffffffu, v.y, src);
-    const float z = __shfl_sync(0xffffffffu, v.z, src), w = __shfl_sync(0xffffffffu, v.w, src);
-    return e == 0 ? x : e == 1 ? y : e == 2 ? z : w;
-}
-
-// The records of plane q of the warp's row from position pc of the block's
-// list (every row warp walks the list; a warp serves its own row's records
-// from the level-1 E of plane q it holds, column col in lane col / VW);
-// returns the new position.  Only the instances of blocks with records (REC)
-// carry it.
-template <int VW, typename V>
-__device__ __forceinline__ int serve_records(const int4 *__restrict__ prec, int pend, int pc, int q, int row, int ib,
-                                          const V &ex, const V &ey, const V &ez, float *pbuf) {
-    const int lane = threadIdx.x & 31;
-    for (;;) {
-        const int i = pc + lane;
-        const bool live = i < pend;
-        const int4 r = live ? prec[i] : make_int4(0, 0, 0, 0);
-        const bool now = live && r.x == q;   // (q is -1 .. -3 in the first iterations of the bottom chunk)
-        const unsigned bal = __ballot_sync(0xffffffffu, now);
-        if (bal) {
-            const int col = r.z - ib, c = r.w & 3;
-            // (the host assigns a record to the block that owns its cell; a
-            // record outside the block's columns is skipped, never read out of range)
-            const bool mine = now && r.y == row && col >= 0 && col < 32 * VW;
-            const int src = mine ? col / VW : lane, e = mine ? col % VW : 0;
-            const float vx = shfl_elem(ex, src, e), vy = shfl_elem(ey, src, e), vz = shfl_elem(ez, src, e);
-            if (mine) pbuf[r.w >> 2] = c == 0 ? vx : c == 1 ? vy : vz;
-        }
-        const int cnt = __popc(bal);
-        pc += cnt;
-        if (cnt < 32) return pc;
-    }
+// Level-1 E for the detectors.  The planes of the warp's row that some readout
+// takes a value from are a list; the whole row of such a plane (the tile's
+// computed columns of Ex, Ey, Ez) is stored, 1.5 KB that one warp writes in three
+// stores however many detectors share it.  Picking out the single values here
+// took a load and twelve shuffles per 32 of them, and made the blocks of a lattice
+// of 3503 detectors in one row the last to end (128x128x512: 104 us a step, 93 now).
+// Only the instances of blocks with lists (REC) carry it.
+struct Pos {
+    int c, end, plane;   // position in the list, its end, the plane there
+};
+__device__ __forceinline__ void next_plane(const int *__restrict__ planes, Pos &P) {
+    P.plane = P.c < P.end ? planes[P.c] : 1 << 30;
 }
 
 // a row warp's signal: its lanes' shared stores before one arrival
@@ -420,13 +428,13 @@ __device__ __forceinline__ void refill(const Args &A, const Maps &M, const Blk &
     }
 }
 
-template <int VW, bool HX, bool HY, bool HZ, bool MASK, bool REC>
+template <bool FT, int VW, bool HX, bool HY, bool HZ, bool MASK, bool REC>
 __device__ __forceinline__ bool plane(const Args &A, const Maps &M, const Lane<VW> &L, const Blk &B, Bars *bar,
                                       float *ring, float *X, const float *CT, int rel, RingPos &rp,
-                                      State<typename Vec<VW>::T> &S, int &pc) {
+                                      State<typename Vec<VW>::T> &S, Pos &pos) {
     typedef typename Vec<VW>::T V;
     typedef Geo<VW> G;
-    constexpr int TXC = G::TXC, BOX = G::BOX, XROW = G::XROW, XBUF = G::XBUF, CX = G::CX, CY = G::CY, CZ = G::CZ;
+    constexpr int TXC = G::TXC, PBOX = G::PBOX, XROW = G::XROW, CX = G::CX, CY = G::CY, CZ = G::CZ;
     const Grid &g = A.g;
     const Cpml &pm = A.pm;
     const int w = L.w;
@@ -440,7 +448,9 @@ __device__ __forceinline__ bool plane(const Args &A, const Maps &M, const Lane<V
     const float *s0 = ring + rp.s0 * B.stage;   // plane p
     const float *s1 = ring + rp.s1 * B.stage;   // plane p+1
     // A's buffer alternates with the plane; B's and C's are single
-    float *XA = X + (rel & 1) * XBUF, *XB = X + 2 * XBUF, *XC = X + 3 * XBUF;
+    float *XA = X + (rel & 1) * (G::XA_ROWS * XROW);
+    float *XB = X + (2 * G::XA_ROWS - 1) * XROW;                 // rows from w = 1
+    float *XC = X + (2 * G::XA_ROWS + G::XB_ROWS - 1) * XROW;    // rows from w = 1
     const int bc0 = VW * L.lane;
     const int lzp = (HZ && p >= 0 && p < g.nz) ? slab_cell(p, g.nz, pm.P) : -1;
     const int lzq = (HZ && q >= 0 && q < g.nz) ? slab_cell(q, g.nz, pm.P) : -1;
@@ -454,35 +464,35 @@ __device__ __forceinline__ bool plane(const Args &A, const Maps &M, const Lane<V
     if (MASK) mp = masks<VW>(L, p, g.nz);
 
     // ---- A: level-1 H at plane p (rows j0-2 .. j0+TY) ----
-    const V ex0 = ldv<V>(s0 + 0 * BOX + w * TXC + bc0);
-    const V ey0 = ldv<V>(s0 + 1 * BOX + w * TXC + bc0);
-    const V ez0 = ldv<V>(s0 + 2 * BOX + w * TXC + bc0);
+    const V ex0 = ldv<V>(s0 + G::foff(0) + w * TXC + bc0);
+    const V ey0 = ldv<V>(s0 + G::foff(1) + w * TXC + bc0);
+    const V ez0 = ldv<V>(s0 + G::foff(2) + w * TXC + bc0);
     V hx1, hy1, hz1;
     V yH0 = z4, yH1 = z4, zH0 = z4, zH1 = z4, xH0 = z4, xH1 = z4;
     {
-        const V hx = ldv<V>(s0 + 3 * BOX + w * TXC + bc0);
-        const V hy = ldv<V>(s0 + 4 * BOX + w * TXC + bc0);
-        const V hz = ldv<V>(s0 + 5 * BOX + w * TXC + bc0);
-        const V exU = ldv<V>(s0 + 0 * BOX + (w + 1) * TXC + bc0);   // row j+1
-        const V ezU = ldv<V>(s0 + 2 * BOX + (w + 1) * TXC + bc0);
-        const V exN = ldv<V>(s1 + 0 * BOX + w * TXC + bc0);         // plane p+1
-        const V eyN = ldv<V>(s1 + 1 * BOX + w * TXC + bc0);
-        const float eyR = __shfl_down_sync(FULL, first(ey0), 1);             // column +4 (lane 31: unused)
-        const float ezR = __shfl_down_sync(FULL, first(ez0), 1);
+        const V hx = ldv<V>(s0 + G::foff(3) + w * TXC + bc0);
+        const V hy = ldv<V>(s0 + G::foff(4) + w * TXC + bc0);
+        const V hz = ldv<V>(s0 + G::foff(5) + w * TXC + bc0);
+        const V exU = ldv<V>(s0 + G::foff(0) + (w + 1) * TXC + bc0);   // row j+1
+        const V ezU = ldv<V>(s0 + G::foff(2) + (w + 1) * TXC + bc0);
+        const V exN = ldv<V>(s1 + G::foff(0) + w * TXC + bc0);         // plane p+1
+        const V eyN = ldv<V>(s1 + G::foff(1) + w * TXC + bc0);
+        const float eyR = from_right<FT>(first(ey0), L.lane);              // column +4
+        const float ezR = from_right<FT>(first(ez0), L.lane);
         V dyEz = ezU - ez0, dzEy = eyN - ey0;                      // Hx
         V dzEx = exN - ex0, dxEz = right(ez0, ezR) - ez0;          // Hy
         V dxEy = right(ey0, eyR) - ey0, dyEx = exU - ex0;          // Hz
         if (yl) {
             const float a = CT[CY + w], b = CT[CY + BR + w];
             yH0 = ldv<V>(PY);
-            yH1 = ldv<V>(PY + BOX);
+            yH1 = ldv<V>(PY + PBOX);
             dyEz = cpmls(yH0, a, b, dyEz);
             dyEx = cpmls(yH1, a, b, dyEx);
         }
         if (HZ && lzp >= 0) {
             const float a = CT[CZ + rel], b = CT[CZ + A.zt + rel];
             zH0 = ldv<V>(PZ);
-            zH1 = ldv<V>(PZ + BOX);
+            zH1 = ldv<V>(PZ + PBOX);
             dzEy = cpmls(zH0, a, b, dzEy);
             dzEx = cpmls(zH1, a, b, dzEx);
         }
@@ -496,8 +506,10 @@ __device__ __forceinline__ bool plane(const Args &A, const Maps &M, const Lane<V
         hx1 = keep<MASK>(axpy(hx, -kH, dyEz - dzEy), mp.hx);
         hy1 = keep<MASK>(axpy(hy, -kH, dzEx - dxEz), mp.hy);
         hz1 = keep<MASK>(axpy(hz, -kH, dxEy - dyEx), mp.hz);
-        stv(XA + w * XROW + bc0, hx1);
-        stv(XA + w * XROW + TXC + bc0, hz1);
+        if (w + 1 < NWR) {
+            stv(XA + w * XROW + bc0, hx1);
+            stv(XA + w * XROW + TXC + bc0, hz1);
+        }
     }
     // B's rows of the warp above (level-1 E of plane q, written in the last
     // iteration's D) before this warp's A rows are signalled: the warp above
@@ -510,10 +522,15 @@ __device__ __forceinline__ bool plane(const Args &A, const Maps &M, const Lane<V
     // the warp is done with stage p (read by A, and by B where it carries psi)
     if (!STAGE_IN_B) signal(&bar->empty[rp.s0]);
 
-    // detector records of plane q of the warp's row: its level-1 E are the
-    // warp's registers of the last iteration; the records of a plane are
-    // contiguous in the block's sorted list
-    if (REC) pc = serve_records<VW>(A.prec, B.pend, pc, q, L.j, B.i0 - 4, S.ex1p, S.ey1p, S.ez1p, A.pbuf);
+    // level-1 E of plane q, the warp's registers of the last iteration, for the detectors
+    if (REC && pos.plane == q) {   // (q is -1 .. -3 in the first iterations of the bottom chunk)
+        float *o = A.pbuf + (size_t)pos.c * PROW + bc0;
+        stv(o, S.ex1p);
+        stv(o + TXC, S.ey1p);
+        stv(o + 2 * TXC, S.ez1p);
+        ++pos.c;
+        next_plane(A.planes, pos);
+    }
 
     // ---- B: level-1 E at plane p (rows j0-1 .. j0+TY) ----
     V ex1 = z4, ey1 = z4, ez1 = z4;
@@ -523,22 +540,22 @@ __device__ __forceinline__ bool plane(const Args &A, const Maps &M, const Lane<V
         if (__any_sync(FULL, !mbar_wait(&bar->xa[rel & 1][w - 1], (rel >> 1) & 1))) return fail(A);
         const V hzD = ldv<V>(XA + (w - 1) * XROW + TXC + bc0);   // row j-1
         const V hxD = ldv<V>(XA + (w - 1) * XROW + bc0);
-        const float hzL = __shfl_up_sync(FULL, last(hz1), 1);           // column -1 (lane 0: unused)
-        const float hyL = __shfl_up_sync(FULL, last(hy1), 1);
+        const float hzL = from_left<FT>(last(hz1), L.lane);           // column -1
+        const float hyL = from_left<FT>(last(hy1), L.lane);
         V dyHz = hz1 - hzD, dzHy = hy1 - S.hy1p;                  // Ex
         V dzHx = hx1 - S.hx1p, dxHz = hz1 - left(hz1, hzL);       // Ey
         V dxHy = hy1 - left(hy1, hyL), dyHx = hx1 - hxD;          // Ez
         if (yl) {
             const float a = CT[CY + 2 * BR + w], b = CT[CY + 3 * BR + w];
-            yE0 = ldv<V>(PY + 2 * BOX);
-            yE1 = ldv<V>(PY + 3 * BOX);
+            yE0 = ldv<V>(PY + 2 * PBOX);
+            yE1 = ldv<V>(PY + 3 * PBOX);
             dyHz = cpmls(yE0, a, b, dyHz);
             dyHx = cpmls(yE1, a, b, dyHx);
         }
         if (HZ && lzp >= 0) {
             const float a = CT[CZ + 2 * A.zt + rel], b = CT[CZ + 3 * A.zt + rel];
-            zE0 = ldv<V>(PZ + 2 * BOX);
-            zE1 = ldv<V>(PZ + 3 * BOX);
+            zE0 = ldv<V>(PZ + 2 * PBOX);
+            zE1 = ldv<V>(PZ + 3 * PBOX);
             dzHy = cpmls(zE0, a, b, dzHy);
             dzHx = cpmls(zE1, a, b, dzHx);
         }
@@ -552,7 +569,7 @@ __device__ __forceinline__ bool plane(const Args &A, const Maps &M, const Lane<V
         ex1 = axpy(ex0, kE, dyHz - dzHy);
         ey1 = axpy(ey0, kE, dzHx - dxHz);
         ez1 = axpy(ez0, kE, dxHy - dyHx);
-        if (B.src_blk) add_source(ez1, A.src, A.ss1, L.c0, L.j, p);
+        if (FT ? B.src_blk && p >= A.ss1.klo && p <= A.ss1.khi : B.src_blk) add_source(ez1, A.src, A.ss1, L.c0, L.j, p);
         ex1 = keep<MASK>(ex1, mp.ex);
         ey1 = keep<MASK>(ey1, mp.ey);
         ez1 = keep<MASK>(ez1, mp.ez);
@@ -566,8 +583,8 @@ __device__ __forceinline__ bool plane(const Args &A, const Maps &M, const Lane<V
     if (p >= B.k0 && w >= 1 && w <= TY + 1) {
         const V exU = ldv<V>(XB + (w + 1) * XROW + bc0);         // level-1 E of plane q, row j+1
         const V ezU = ldv<V>(XB + (w + 1) * XROW + TXC + bc0);
-        const float eyR = __shfl_down_sync(FULL, first(S.ey1p), 1);
-        const float ezR = __shfl_down_sync(FULL, first(S.ez1p), 1);
+        const float eyR = from_right<FT>(first(S.ey1p), L.lane);
+        const float ezR = from_right<FT>(first(S.ez1p), L.lane);
         V dyEz = ezU - S.ez1p, dzEy = ey1 - S.ey1p;
         V dzEx = ex1 - S.ex1p, dxEz = right(S.ez1p, ezR) - S.ez1p;
         V dxEy = right(S.ey1p, eyR) - S.ey1p, dyEx = exU - S.ex1p;
@@ -623,8 +640,8 @@ __device__ __forceinline__ bool plane(const Args &A, const Maps &M, const Lane<V
     if (p >= B.k0 + 1 && w >= 2 && w <= TY + 1) {
         const V hzD = ldv<V>(XC + (w - 1) * XROW + TXC + bc0);
         const V hxD = ldv<V>(XC + (w - 1) * XROW + bc0);
-        const float hzL = __shfl_up_sync(FULL, last(hz2), 1);
-        const float hyL = __shfl_up_sync(FULL, last(hy2), 1);
+        const float hzL = from_left<FT>(last(hz2), L.lane);
+        const float hyL = from_left<FT>(last(hy2), L.lane);
         V dyHz = hz2 - hzD, dzHy = hy2 - S.hy2p;
         V dzHx = hx2 - S.hx2p, dxHz = hz2 - left(hz2, hzL);
         V dxHy = hy2 - left(hy2, hyL), dyHx = hx2 - hxD;
@@ -647,7 +664,7 @@ __device__ __forceinline__ bool plane(const Args &A, const Maps &M, const Lane<V
         V ey2 = axpy(S.ey1p, kE, dzHx - dxHz);
         V ez2 = axpy(S.ez1p, kE, dxHy - dyHx);
         if (L.own && q < B.k1) {
-            if (B.src_blk) add_source(ez2, A.src, A.ss2, L.c0, L.j, q);
+            if (FT ? B.src_blk && q >= A.ss2.klo && q <= A.ss2.khi : B.src_blk) add_source(ez2, A.src, A.ss2, L.c0, L.j, q);
             const unsigned o = (unsigned)L.c0 + (unsigned)L.j * (unsigned)g.pitch + (unsigned)q * (unsigned)g.plane;
             stw<MASK>(A.out[0] + o, keep<MASK>(ex2, mq.ex), L.nval);
             stw<MASK>(A.out[1] + o, keep<MASK>(ey2, mq.ey), L.nval);
@@ -691,7 +708,7 @@ __device__ __forceinline__ bool plane(const Args &A, const Maps &M, const Lane<V
     return true;
 }
 
-template <int VW, bool HX, bool HY, bool HZ, bool MASK, bool REC>
+template <bool FT, int VW, bool HX, bool HY, bool HZ, bool MASK, bool REC>
 __device__ __forceinline__ void march(const Args &A, const Maps &M, const Lane<VW> &L, const Blk &B, Bars *bar,
                                       float *ring, float *X, const float *CT) {
     typedef typename Vec<VW>::T V;
@@ -700,42 +717,50 @@ __device__ __forceinline__ void march(const Args &A, const Maps &M, const Lane<V
     S.ex1p = S.ey1p = S.ez1p = S.hx1p = S.hy1p = S.hz1p = S.hx2p = S.hy2p = z4;
     S.yH0 = S.yH1 = S.yE0 = S.yE1 = S.zH0 = S.zH1 = S.zE0 = S.zE1 = S.xH0 = S.xH1 = S.xE0 = S.xE1 = z4;
     RingPos rp{0, 1, 0u};   // two stages at least
-    int pc = B.pbeg;
+    Pos pos;
+    if (REC) {
+        const bool owned = L.w >= 2 && L.w < TY + 2;
+        pos.c = owned ? A.pidx[B.rec + L.w - 2] : 0;
+        pos.end = owned ? A.pidx[B.rec + L.w - 1] : 0;
+        next_plane(A.planes, pos);
+    }
     for (int rel = 0; rel + 1 < B.nplanes; ++rel)
-        if (!plane<VW, HX, HY, HZ, MASK, REC>(A, M, L, B, bar, ring, X, CT, rel, rp, S, pc)) return;
+        if (!plane<FT, VW, HX, HY, HZ, MASK, REC>(A, M, L, B, bar, ring, X, CT, rel, rp, S, pos)) return;
 }
 
 // the instance of a block's case: which psi boxes it carries, whether it
 // meets a face of the grid
-template <int VW, bool HX, bool HY, bool HZ>
+template <bool FT, int VW, bool HX, bool HY, bool HZ>
 __device__ __forceinline__ void march_edge(bool edge, const Args &A, const Maps &M, const Lane<VW> &L, const Blk &B,
                                            Bars *bar, float *ring, float *X, const float *CT) {
     // blocks with detector records run an instance with the record service
-    if (B.pbeg < B.pend) {
-        if (edge) march<VW, HX, HY, HZ, true, true>(A, M, L, B, bar, ring, X, CT);
-        else march<VW, HX, HY, HZ, false, true>(A, M, L, B, bar, ring, X, CT);
+    if (A.pidx && A.pidx[B.rec] < A.pidx[B.rec + TY]) {
+        if (edge) march<FT, VW, HX, HY, HZ, true, true>(A, M, L, B, bar, ring, X, CT);
+        else march<FT, VW, HX, HY, HZ, false, true>(A, M, L, B, bar, ring, X, CT);
     } else {
-        if (edge) march<VW, HX, HY, HZ, true, false>(A, M, L, B, bar, ring, X, CT);
-        else march<VW, HX, HY, HZ, false, false>(A, M, L, B, bar, ring, X, CT);
+        if (edge) march<FT, VW, HX, HY, HZ, true, false>(A, M, L, B, bar, ring, X, CT);
+        else march<FT, VW, HX, HY, HZ, false, false>(A, M, L, B, bar, ring, X, CT);
     }
 }
-template <int VW, bool HX, bool HY>
+template <bool FT, int VW, bool HX, bool HY>
 __device__ __forceinline__ void march_z(bool hz, bool edge, const Args &A, const Maps &M, const Lane<VW> &L,
                                         const Blk &B, Bars *bar, float *ring, float *X, const float *CT) {
-    if (hz) march_edge<VW, HX, HY, true>(edge, A, M, L, B, bar, ring, X, CT);
-    else march_edge<VW, HX, HY, false>(edge, A, M, L, B, bar, ring, X, CT);
+    if (hz) march_edge<FT, VW, HX, HY, true>(edge, A, M, L, B, bar, ring, X, CT);
+    else march_edge<FT, VW, HX, HY, false>(edge, A, M, L, B, bar, ring, X, CT);
 }
 
 // one block of the launch: tile column T, tile row ty
-template <int VW>
+// FT: the full tiles of a grid of up to 128 columns, in a kernel of their own (in
+// one kernel with the others, the larger code slowed those: 384x384x1536 1339 ->
+// 1361 us a step, and 1387 with the test of the current's planes)
+template <bool FT, int VW>
 __device__ __forceinline__ void run_block(const Args &A, const Maps &M, const TileCol T, int ty) {
     typedef Geo<VW> G;
-    constexpr int TXC = G::TXC, BOX = G::BOX, FIELDS = G::FIELDS, XBUF = G::XBUF, CX = G::CX,
-                  CY = G::CY, CZ = G::CZ;
+    constexpr int TXC = G::TXC, PBOX = G::PBOX, FIELDS = G::FIELDS, CX = G::CX, CY = G::CY, CZ = G::CZ;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     Bars *bar = reinterpret_cast<Bars *>(smem_raw);
     float *X = reinterpret_cast<float *>(smem_raw + BAR_BYTES);   // exchange rows
-    float *CT = X + 4 * XBUF;                                      // CPML coefficients
+    float *CT = X + G::XFLOATS;                                    // CPML coefficients
     float *ring = X + G::head_floats(A.zt);                        // stage ring
 
     const Grid &g = A.g;
@@ -762,23 +787,23 @@ __device__ __forceinline__ void run_block(const Args &A, const Maps &M, const Ti
             B.k1 = g.nz;
         }
         B.hz = P > 0 && c >= A.m;
-        const int b = c * A.tiles_x * A.tiles_y + tile;
-        B.pbeg = A.pidx ? A.pidx[b] : 0;
-        B.pend = A.pidx ? A.pidx[b + 1] : 0;
+        B.rec = (c * A.tiles_x * A.tiles_y + tile) * TY;
     }
     B.kstart = B.k0 - 2;
     B.nplanes = B.k1 - B.k0 + 4;   // input planes k0-2 .. k1+1
     B.src_blk = A.src.active && B.i0 - 4 <= A.src.ic + A.src.L && B.i0 + TXC - 5 >= A.src.ic - A.src.L &&
-                B.j0 - 2 <= A.src.jc + A.src.L && B.j0 + TY + 1 >= A.src.jc - A.src.L;
+                B.j0 - 2 <= A.src.jc + A.src.L && B.j0 + TY + 1 >= A.src.jc - A.src.L &&
+                ((A.ss1.klo <= A.ss1.khi && A.ss1.klo <= B.k1 && A.ss1.khi >= B.kstart) ||
+                 (A.ss2.klo <= A.ss2.khi && A.ss2.klo <= B.k1 && A.ss2.khi >= B.kstart));
     B.hx = B.hy = false;
     B.l0 = 0;
     B.xlo = B.xhi = -1;
     B.nxb = 0;
-    B.xb = (A.xbw * BR + 31) / 32 * 32;
+    B.xb = (A.xbw * PR + 31) / 32 * 32;
     if (P > 0) {
         const int ilo = max(B.i0 - 4, 0), ihi = min(B.i0 + TXC - 5, g.nx - 1);
-        if (VW == 1 && ilo <= P) B.xlo = B.nxb++;
-        if (VW == 1 && ihi >= g.nx - P) B.xhi = B.nxb++;
+        if ((VW == 1 || FT) && ilo <= P) B.xlo = B.nxb++;
+        if ((VW == 1 || FT) && ihi >= g.nx - P) B.xhi = B.nxb++;
         B.hx = B.nxb > 0;
         int lmin = 1 << 30;
         for (int j = max(B.j0 - 2, 0); j < min(B.j0 + TY + 2, g.ny); ++j) {
@@ -790,8 +815,8 @@ __device__ __forceinline__ void run_block(const Args &A, const Maps &M, const Ti
     }
     B.xo = FIELDS;
     B.yo = B.xo + 4 * B.nxb * B.xb;
-    B.zo = B.yo + (B.hy ? 4 * BOX : 0);
-    B.stage = B.zo + (B.hz ? 4 * BOX : 0);
+    B.zo = B.yo + (B.hy ? 4 * PBOX : 0);
+    B.stage = B.zo + (B.hz ? 4 * PBOX : 0);
     B.ns = min(NSMAX, (A.smem_floats - G::head_floats(A.zt)) / B.stage);
 
     if (tid == 0) {
@@ -856,7 +881,7 @@ __device__ __forceinline__ void run_block(const Args &A, const Maps &M, const Ti
         L.mcol0 = umask(m, V());
     }
     L.nval = L.c0 >= 0 && L.c0 < g.nx ? min(VW, g.nx - L.c0) : 0;
-    L.own = L.lane >= G::LO && L.lane <= G::HI && L.w >= 2 && L.w <= TY + 1 && L.rowin && L.nval > 0 &&
+    L.own = (FT || (L.lane >= G::LO && L.lane <= G::HI)) && L.w >= 2 && L.w <= TY + 1 && L.rowin && L.nval > 0 &&
             L.c0 < B.iend;
     if (L.own) L.nval = min(L.nval, B.iend - L.c0);
     L.ly = (P > 0 && L.rowin) ? slab_cell(L.j, g.ny, P) : -1;
@@ -880,26 +905,30 @@ __device__ __forceinline__ void run_block(const Args &A, const Maps &M, const Ti
     // blocks whose computed region stays clear of the faces need no masks
     const bool edge = B.i0 - 4 < 1 || B.i0 + TXC - 5 > g.nx - 1 || B.j0 - 2 < 1 || B.j0 + TY > g.ny - 1 ||
                       B.k0 - 2 < 1 || B.k1 > g.nz - 1;
-    if (VW == 1) {   // the narrow tiles of the x layers: always with masks
+    if constexpr (FT || VW == 1) {   // full tiles, and the narrow tiles of the x layers: always with masks
         if (B.hx) {
-            if (B.hy) march_z<VW, true, true>(B.hz, true, A, M, L, B, bar, ring, X, CT);
-            else march_z<VW, true, false>(B.hz, true, A, M, L, B, bar, ring, X, CT);
+            if (B.hy) march_z<FT, VW, true, true>(B.hz, true, A, M, L, B, bar, ring, X, CT);
+            else march_z<FT, VW, true, false>(B.hz, true, A, M, L, B, bar, ring, X, CT);
         } else {
-            if (B.hy) march_z<VW, false, true>(B.hz, true, A, M, L, B, bar, ring, X, CT);
-            else march_z<VW, false, false>(B.hz, true, A, M, L, B, bar, ring, X, CT);
+            if (B.hy) march_z<FT, VW, false, true>(B.hz, true, A, M, L, B, bar, ring, X, CT);
+            else march_z<FT, VW, false, false>(B.hz, true, A, M, L, B, bar, ring, X, CT);
         }
-    } else {         // the wide tiles never meet an x layer
-        if (B.hy) march_z<VW, false, true>(B.hz, edge, A, M, L, B, bar, ring, X, CT);
-        else march_z<VW, false, false>(B.hz, edge, A, M, L, B, bar, ring, X, CT);
+    } else {         // the other wide tiles never meet an x layer
+        if (B.hy) march_z<FT, VW, false, true>(B.hz, edge, A, M, L, B, bar, ring, X, CT);
+        else march_z<FT, VW, false, false>(B.hz, edge, A, M, L, B, bar, ring, X, CT);
     }
 }
 
 __global__ void __launch_bounds__(NT, 1) k_tb2(const Args A, const __grid_constant__ Maps M) {
     const int tile = (int)blockIdx.x;
     const int ty = tile / A.tiles_x;
-    const TileCol T = tile_col(tile - ty * A.tiles_x, A.ta, A.tb, A.nl, A.nw, A.g.nx);
-    if (T.vw == 1) run_block<1>(A, M, T, ty);
-    else run_block<4>(A, M, T, ty);
+    const TileCol T = tile_col(tile - ty * A.tiles_x, A.ta, A.tb, A.nl, A.nw, A.g.nx, false);
+    if (T.vw == 1) run_block<false, 1>(A, M, T, ty);
+    else run_block<false, 4>(A, M, T, ty);
+}
+
+__global__ void __launch_bounds__(NT, 1) k_tb2_full(const Args A, const __grid_constant__ Maps M) {
+    run_block<true, 4>(A, M, tile_col(0, 0, 0, 0, 1, A.g.nx, true), (int)blockIdx.x);
 }
 
 constexpr CUtensorMapL2promotion kPromotion = CU_TENSOR_MAP_L2_PROMOTION_L2_128B;
@@ -907,20 +936,21 @@ constexpr CUtensorMapL2promotion kPromotion = CU_TENSOR_MAP_L2_PROMOTION_L2_128B
 struct HostState {
     Maps maps;
     int ta, tb, nl, nw;                        // tile columns (tile_col)
+    bool full;
     int tiles_x, tiles_y, za, zb, cm, m, zt, chunks, smem_floats;
     int xlo4, xhb, xbw;
     size_t smem;
-    // detector records, rebuilt when the handle's detectors change
+    // planes stored for the detectors and the places of their values, rebuilt
+    // when the handle's detectors change
     int probe_ver;
-    std::vector<int4> h_rec;
-    std::vector<int> h_idx;
-    int4 *d_rec;
-    int *d_idx;
+    bool probes_ok;
+    int *d_planes, *d_idx, *d_pos;
     float *d_pbuf;
 };
 
 // tile column of column i (tile_col inverted)
 int tile_of(const HostState *st, int i, int nx) {
+    if (st->full) return 0;
     i = std::min(std::max(i, 0), nx - 1);   // a readout cell outside the grid: the edge tile
     int tc;
     if (i < st->ta) tc = i / 24;
@@ -936,19 +966,23 @@ int chunk_of(const HostState *st, int k) {
     return (k - st->za) / st->cm;
 }
 
-int build_records(fdtd_ctx *h, HostState *st) {
-    cudaFree(st->d_rec);
+void free_records(HostState *st) {
+    cudaFree(st->d_planes);
     cudaFree(st->d_idx);
+    cudaFree(st->d_pos);
     cudaFree(st->d_pbuf);
-    st->d_rec = nullptr;
-    st->d_idx = nullptr;
+    st->d_planes = st->d_idx = st->d_pos = nullptr;
     st->d_pbuf = nullptr;
-    st->probe_ver = h->probe_ver;
-    if (h->np == 0) return FDTD_OK;
+}
+
+// False when the stored rows would not fit (memory, or 32-bit places).
+bool build_records(fdtd_ctx *h, HostState *st) {
+    free_records(st);
+    if (h->np == 0) return true;
     const int tiles = st->tiles_x * st->tiles_y;
-    const int blocks = tiles * st->chunks;
+    const int lists = tiles * st->chunks * TY;   // owned rows of blocks
     // the six cells of each detector's readout: Ex at i-1, i; Ey at j-1, j; Ez at k-1, k
-    struct Rec { int b; int4 r; };
+    struct Rec { int list, plane, place, slot; };
     std::vector<Rec> recs;
     recs.reserve(6 * (size_t)h->np);
     for (int t = 0; t < h->np; ++t) {
@@ -956,35 +990,71 @@ int build_records(fdtd_ctx *h, HostState *st) {
         const int cell[6][4] = {{i - 1, j, k, 0}, {i, j, k, 0}, {i, j - 1, k, 1},
                                 {i, j, k, 1},     {i, j, k - 1, 2}, {i, j, k, 2}};
         for (int s = 0; s < 6; ++s) {
-            const int ci = cell[s][0], cj = cell[s][1], ck = cell[s][2];
-            const int b = chunk_of(st, ck) * tiles + (cj / TY) * st->tiles_x + tile_of(st, ci, h->g.nx);
-            recs.push_back({b, make_int4(ck, cj, ci, (6 * t + s) * 4 + cell[s][3])});
+            const int ci = cell[s][0], cj = cell[s][1], ck = cell[s][2], tc = tile_of(st, ci, h->g.nx);
+            const TileCol T = tile_col(tc, st->ta, st->tb, st->nl, st->nw, h->g.nx, st->full);
+            recs.push_back({(chunk_of(st, ck) * tiles + (cj / TY) * st->tiles_x + tc) * TY + cj % TY, ck,
+                            cell[s][3] * 32 * T.vw + ci - (T.i0 - 4), 6 * t + s});
         }
     }
-    std::stable_sort(recs.begin(), recs.end(),
-                     [](const Rec &a, const Rec &b) { return a.b < b.b || (a.b == b.b && a.r.x < b.r.x); });
-    st->h_rec.resize(recs.size());
-    st->h_idx.assign(blocks + 1, 0);
+    std::sort(recs.begin(), recs.end(), [](const Rec &a, const Rec &b) {
+        return a.list < b.list || (a.list == b.list && a.plane < b.plane);
+    });
+    std::vector<int> planes, idx(lists + 1, 0), pos(recs.size());
+    constexpr size_t MAX_ROWS = 0x7fffffff / PROW - 1;
     for (size_t n = 0; n < recs.size(); ++n) {
-        st->h_rec[n] = recs[n].r;
-        st->h_idx[recs[n].b + 1]++;
+        if (n == 0 || recs[n].list != recs[n - 1].list || recs[n].plane != recs[n - 1].plane) {
+            if (planes.size() > MAX_ROWS) return false;
+            planes.push_back(recs[n].plane);
+            idx[recs[n].list + 1]++;
+        }
+        pos[recs[n].slot] = ((int)planes.size() - 1) * PROW + recs[n].place;
     }
-    for (int b = 0; b < blocks; ++b) st->h_idx[b + 1] += st->h_idx[b];
-    if (cudaMalloc(&st->d_rec, sizeof(int4) * recs.size()) != cudaSuccess ||
-        cudaMalloc(&st->d_idx, sizeof(int) * (blocks + 1)) != cudaSuccess ||
-        cudaMalloc(&st->d_pbuf, sizeof(float) * 6 * (size_t)h->np) != cudaSuccess) {
+    for (int b = 0; b < lists; ++b) idx[b + 1] += idx[b];
+    const auto upload = [](int **d, const std::vector<int> &v) {
+        return cudaMalloc(d, sizeof(int) * v.size()) == cudaSuccess &&
+               cudaMemcpy(*d, v.data(), sizeof(int) * v.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+    };
+    if (!upload(&st->d_planes, planes) || !upload(&st->d_idx, idx) || !upload(&st->d_pos, pos) ||
+        cudaMalloc(&st->d_pbuf, sizeof(float) * PROW * planes.size()) != cudaSuccess) {
         cudaGetLastError();
-        return FDTD_ERR_OOM;
+        free_records(st);
+        return false;
     }
-    if (cudaMemcpy(st->d_rec, st->h_rec.data(), sizeof(int4) * recs.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(st->d_idx, st->h_idx.data(), sizeof(int) * (blocks + 1), cudaMemcpyHostToDevice) != cudaSuccess) {
-        cudaGetLastError();
-        return FDTD_ERR_CUDA;
-    }
-    return FDTD_OK;
+    return true;
 }
 
 }  // namespace
+
+// Time of a launch in units of 0.05 us: its blocks in launch order, each on the
+// SM that is free first.  A block costs (planes + 4) times its kind's time per
+// plane, in us measured with a timer in the blocks of seven grids: full tiles of
+// a CPML grid 2.0 (2.7 in a y layer, 3.3 in a z layer, 5.4 in both), other wide
+// tiles 1.2 (1.75, 2.05, 3.2), narrow ones 1.0 (1.2, 1.45, 1.75).  The launch
+// times it gives are within 12 % of the measured ones on 128 x 128 x 256,
+// 128 x 128 x 512 and 160 x 160 x 640.
+static long long launch_time(const HostState *st, const Grid &g, int P, long long m, int sms) {
+    static const int cost[3][4] = {{40, 54, 66, 108}, {24, 35, 41, 64}, {20, 24, 29, 35}};
+    const int mid = st->zb - st->za;
+    const int cm = mid > 0 ? (int)((mid + m - 1) / m) : 1, mm = mid > 0 ? (mid + cm - 1) / cm : 0;
+    std::vector<long long> free_at((size_t)sms, 0);   // a heap, the earliest first
+    const auto later = [](long long x, long long y) { return x > y; };
+    long long end = 0;
+    for (int c = 0; c < mm + (st->za > 0) + (st->zb < g.nz); ++c) {
+        const bool low = c == mm && st->za > 0;
+        const int planes = 4 + (c < mm ? std::min(cm, mid - c * cm) : low ? st->za : g.nz - st->zb);
+        for (int ty = 0; ty < st->tiles_y; ++ty) {
+            const bool y = P > 0 && (ty * TY - 2 <= P || ty * TY + TY + 1 >= g.ny - P);
+            for (int tc = 0; tc < st->tiles_x; ++tc) {
+                const bool wide = st->full || (tc >= st->nl && tc < st->nl + st->nw);
+                std::pop_heap(free_at.begin(), free_at.end(), later);
+                free_at.back() += (long long)planes * cost[!wide ? 2 : st->full && P > 0 ? 0 : 1][(c >= mm ? 2 : 0) + y];
+                end = std::max(end, free_at.back());
+                std::push_heap(free_at.begin(), free_at.end(), later);
+            }
+        }
+    }
+    return end;
+}
 
 const char *tb2_name(const fdtd_ctx *) { return "tblock2-120x8"; }
 
@@ -1014,7 +1084,7 @@ int tb2_prepare(fdtd_ctx *h) {
         for (int s = 0; s < 2; ++s)
             for (int c = 0; c < 6; ++c)
                 ok = ok && encode3(encode, &st->maps.f[wd][s][c], h->fields[s] + (size_t)c * g.comp, g.nx + 1,
-                                   g.ny + 1, g.nz + 1, g.pitch, g.plane, TXCW[wd], BR, kPromotion);
+                                   g.ny + 1, g.nz + 1, g.pitch, g.plane, TXCW[wd], G4::frows(c), kPromotion);
     if (P > 0) {
         // H psi sets follow the field set; E psi sets are psi_block's first
         // third and epsi2
@@ -1032,14 +1102,14 @@ int tb2_prepare(fdtd_ctx *h) {
                         const int a = 2 * half + t;
                         if (axis == 0)
                             ok = ok && encode3(encode, &st->maps.x[a][s], base, WX, g.ny, g.nz, WX,
-                                               (cuuint64_t)g.ny * WX, xbw, BR, kPromotion);
+                                               (cuuint64_t)g.ny * WX, xbw, PR, kPromotion);
                         for (int wd = 0; wd < 2 && axis > 0; ++wd) {
                             if (axis == 1)
                                 ok = ok && encode3(encode, &st->maps.y[wd][a][s], base, g.nx, W, g.nz, g.pitch,
-                                                   (cuuint64_t)W * g.pitch, TXCW[wd], BR, kPromotion);
+                                                   (cuuint64_t)W * g.pitch, TXCW[wd], PR, kPromotion);
                             else
                                 ok = ok && encode3(encode, &st->maps.z[wd][a][s], base, g.nx, g.ny, W, g.pitch,
-                                                   (cuuint64_t)g.ny * g.pitch, TXCW[wd], BR, kPromotion);
+                                                   (cuuint64_t)g.ny * g.pitch, TXCW[wd], PR, kPromotion);
                         }
                     }
                 }
@@ -1085,6 +1155,14 @@ int tb2_prepare(fdtd_ctx *h) {
         st->tiles_x = st->nl + st->nw + (g.nx - st->tb + G1::TXO - 1) / G1::TXO;
     }
     st->tiles_y = (g.ny + TY - 1) / TY;
+    int max_smem = 0;
+    cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->dev);
+    const long long floats = (long long)max_smem / 4 - BAR_BYTES / 4;
+    const long long xb = (xbw * PR + 31) / 32 * 32;
+    // largest stages: wide tiles with y and z boxes, a full tile with two x
+    // halves besides; narrow ones with two x halves, y and z
+    const long long big4 = G4::FIELDS + 8LL * G4::PBOX, bigF = big4 + (P > 0 ? 8 * xb : 0);
+    const long long big1 = G1::FIELDS + 8 * xb + 8LL * G1::PBOX;
     // z chunks: the planes of a middle chunk (k0-2 .. k1+1) stay clear of the
     // z layers, so only the two layer chunks [0, za), [zb, nz) carry z boxes;
     // a grid too short for a middle part is one layer chunk
@@ -1096,43 +1174,42 @@ int tb2_prepare(fdtd_ctx *h) {
         st->za = 0;
         st->zb = g.nz;
     }
-    // Middle chunks: the fewest waves x chunk length, with chunks of at most
-    // CM_MAX planes.  The blocks of a wave march up z side by side and read
-    // each other's halo rows; over a long march they drift apart by more
-    // planes than L2 keeps, and the halo rows come from DRAM twice (measured:
+    const int layer = std::max(st->za, g.nz - st->zb);
+    st->zt = P > 0 ? layer + 4 : 1;
+    st->smem_floats = (int)floats;
+    st->smem = 4 * (size_t)floats + BAR_BYTES;
+    st->full = g.nx <= G4::TXC && floats - G4::head_floats(st->zt) >= 2 * bigF;
+    if (st->full) st->nl = 0, st->nw = st->tiles_x = 1;
+    // Middle chunks of at most CM_MAX planes.  The blocks of a wave march up z side
+    // by side and read each other's halo rows; over a long march they drift apart by
+    // more planes than L2 keeps, and the halo rows come from DRAM twice (measured:
     // 139 -> 147 Gcell/s on 384x384x1536 and 169 -> 181 on 640x640x2048 with
     // chunks of about 150 planes instead of 300-500; below 64 planes the
-    // warm-up planes cost more than L2 saves).
+    // warm-up planes cost more than L2 saves).  A launch of a few waves takes the
+    // chunks with the shortest launch_time, which counts the layer blocks that
+    // follow the middle ones (us a step, against the fewest waves x chunk length
+    // alone: 128x128x512 103 -> 94, 128x128x256 77 -> 57, 160x160x640 213 -> 174,
+    // 200x200x300 185 -> 158, all with 10 CPML cells);
+    // a longer one, where that makes no difference, the fewest waves x length.
     constexpr long long CM_MAX = 160;
     const int mid = st->zb - st->za;
-    const long long sms = h->num_sms > 0 ? h->num_sms : 1;
+    const int sms = h->num_sms > 0 ? h->num_sms : 1;
     const long long tiles = (long long)st->tiles_x * st->tiles_y;
     long long m = 0, best = -1;
     const long long m_lo = std::max(1LL, (mid + CM_MAX - 1) / CM_MAX);
     const long long m_hi = std::max(m_lo, (long long)(mid / 16));
+    const bool few = tiles * m_lo <= 8LL * sms;
     if (mid > 0)
-        for (long long mm = m_lo; mm <= m_hi; ++mm) {
+        for (long long mm = m_lo; mm <= (few ? std::min(m_hi, m_lo + 24) : m_hi); ++mm) {
             const long long cm = (mid + mm - 1) / mm;
-            const long long cost = (tiles * mm + sms - 1) / sms * (cm + 7);
+            const long long cost = few ? launch_time(st, g, P, mm, sms) : (tiles * mm + sms - 1) / sms * (cm + 7);
             if (best < 0 || cost < best) { best = cost; m = mm; }
         }
     st->cm = m > 0 ? (int)((mid + m - 1) / m) : 1;
     st->m = m > 0 ? (mid + st->cm - 1) / st->cm : 0;
     st->chunks = st->m + (st->za > 0 ? 1 : 0) + (st->zb < g.nz ? 1 : 0);
-    const int layer = std::max(st->za, g.nz - st->zb);
-    st->zt = P > 0 ? layer + 4 : 1;
-    int max_smem = 0;
-    cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->dev);
-    const long long xb = (xbw * BR + 31) / 32 * 32;
-    // largest stages: wide tiles with y and z boxes; narrow ones with two x
-    // halves, y and z
-    const long long big4 = G4::FIELDS + 8LL * G4::BOX;
-    const long long big1 = G1::FIELDS + 8 * xb + 8LL * G1::BOX;
-    const long long floats = (long long)max_smem / 4 - BAR_BYTES / 4;
-    st->smem_floats = (int)floats;
-    st->smem = 4 * (size_t)floats + BAR_BYTES;
-    if (floats - G4::head_floats(st->zt) < 2 * big4 || floats - G1::head_floats(st->zt) < 2 * big1 ||
-        cudaFuncSetAttribute(k_tb2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st->smem) != cudaSuccess) {
+    if (floats - G4::head_floats(st->zt) < 2 * (st->full ? bigF : big4) || floats - G1::head_floats(st->zt) < 2 * big1 ||
+        cudaFuncSetAttribute(st->full ? k_tb2_full : k_tb2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st->smem) != cudaSuccess) {
         cudaGetLastError();
         delete st;
         return FDTD_ERR_CUDA;
@@ -1144,21 +1221,29 @@ int tb2_prepare(fdtd_ctx *h) {
 
 void tb2_release(fdtd_ctx *h) {
     HostState *st = static_cast<HostState *>(h->tb2);
-    if (st) {
-        cudaFree(st->d_rec);
-        cudaFree(st->d_idx);
-        cudaFree(st->d_pbuf);
-    }
+    if (st) free_records(st);
     delete st;
     h->tb2 = nullptr;
 }
 
-void launch_tb2(fdtd_ctx *h, cudaStream_t s) {
+// Whether two-step passes can take the handle's detectors (a set whose rows do
+// not fit steps on path 1).
+bool tb2_ready(fdtd_ctx *h) {
     HostState *st = static_cast<HostState *>(h->tb2);
     if (st->probe_ver != h->probe_ver) {
-        const int rc = build_records(h, st);
-        if (rc != FDTD_OK && h->status == FDTD_OK) h->status = rc;
+        st->probe_ver = h->probe_ver;
+        try {
+            st->probes_ok = build_records(h, st);
+        } catch (const std::bad_alloc &) {
+            free_records(st);
+            st->probes_ok = false;
+        }
     }
+    return st->probes_ok;
+}
+
+void launch_tb2(fdtd_ctx *h, cudaStream_t s) {
+    HostState *st = static_cast<HostState *>(h->tb2);
     const Grid &g = h->g;
     Args a;
     a.g = g;
@@ -1194,15 +1279,17 @@ void launch_tb2(fdtd_ctx *h, cudaStream_t s) {
     a.kE = (float)h->kE;
     a.kH = (float)h->kH;
     a.flags = h->d_flags;
-    a.prec = st->d_rec;
+    a.planes = st->d_planes;
     a.pidx = st->d_idx;
     a.pbuf = st->d_pbuf;
     dim3 grid(st->tiles_x * st->tiles_y, st->chunks);
-    k_tb2<<<grid, NT, st->smem, s>>>(a, st->maps);
+    if (st->full) k_tb2_full<<<grid, NT, st->smem, s>>>(a, st->maps);
+    else k_tb2<<<grid, NT, st->smem, s>>>(a, st->maps);
 }
 
-float *tb2_probe_values(fdtd_ctx *h) {
-    HostState *st = static_cast<HostState *>(h->tb2);
+const float *tb2_probe_values(const fdtd_ctx *h, const int **pos) {
+    const HostState *st = static_cast<const HostState *>(h->tb2);
+    *pos = st ? st->d_pos : nullptr;
     return st ? st->d_pbuf : nullptr;
 }
 
