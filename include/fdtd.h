@@ -229,9 +229,9 @@ const char *fdtd_kernel_name(fdtd_t h);
  *       grids only (FDTD_ERR_ARG on a Mur grid).  The default of PEC grids
  *       that do not fit the resident runs of path 1 (100^3: 20.7 -> 18.6 us a
  *       step), of CPML grids of up to 128 columns from 2.5 million cells
- *       (128 x 128 x 512, CPML 10: 124 -> 93; 128^3: 49 against 52) and of
+ *       (128 x 128 x 512, CPML 10: 124 -> 79; 128^3: 49 against 52) and of
  *       other CPML grids from FDTD_TWO_STEP_MIN_CELLS cells, about 12.6 million
- *       (160 x 160 x 640: 274 -> 174; 200^3: 116 against 117.5);
+ *       (160 x 160 x 640: 274 -> 173; 200^3: 116 against 117.5);
  *   1 = one pass per step: TMA-staged vector-tile z-march over the whole
  *       grid, CPML included (the default on Mur grids and smaller grids).
  *       Runs of two steps or more of a small PEC or Mur grid (nx <= 127, and

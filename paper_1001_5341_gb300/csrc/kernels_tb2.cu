@@ -10,7 +10,7 @@
 // A grid of up to 128 columns is one wide tile of all its columns, x layers
 // included (nothing lies beyond its ends, so it needs no halo there): with a wide
 // tile between two narrow ones 128x128x512 (10 CPML cells) took 144 us a step,
-// with one full tile 106 (93 with the chunks of launch_time); PEC 90 -> 46.
+// with one full tile 106 (79 with the chunks of launch_time); PEC 90 -> 45.
 //
 // Tiles.  A wide block owns up to 120 columns [i0, i0+120) by TY = 8 rows
 // [j0, j0+8) and marches up a chunk of z planes [k0, k1).  It computes the
@@ -249,13 +249,60 @@ __host__ __device__ inline TileCol tile_col(int tc, int a, int b, int nl, int nw
     return t;
 }
 
+// The blocks of a launch: the middle planes [za, zb) in m chunks of cm planes, in
+// the `ry` tile rows of the y layers (rl of them low) my chunks of cy, then the two
+// layer chunks [0, za), [zb, nz) of every tile.  Numbered chunk by chunk, so that
+// the tiles of a chunk start together.  (A table of blocks in memory would do, but
+// then the block's geometry no longer lies in uniform registers: 384x384x1536 1340
+// -> 1362 us a step.)
+struct Cut {
+    int tiles_x, tiles_y, ry, rl, za, zb, nz, m, cm, my, cy;
+    int layer;              // whether the outer chunks are CPML layers (z boxes)
+    __host__ __device__ int mid_blocks() const { return m * tiles_x * (tiles_y - ry); }
+    __host__ __device__ int y_blocks() const { return my * tiles_x * ry; }
+    __host__ __device__ int blocks() const {
+        return mid_blocks() + y_blocks() + tiles_x * tiles_y * ((za > 0) + (zb < nz));
+    }
+};
+struct Item {
+    int tc, ty, k0, k1, hz;
+};
+__host__ __device__ __forceinline__ Item item(const Cut &c, int b) {
+    Item t;
+    const int nm = c.mid_blocks(), n = nm + c.y_blocks();
+    if (b < nm) {
+        const int rows = c.tiles_y - c.ry, per = c.tiles_x * rows, q = b / per, e = b - q * per;
+        t.ty = c.rl + e / c.tiles_x;
+        t.tc = e % c.tiles_x;
+        t.k0 = c.za + q * c.cm;
+        t.k1 = t.k0 + c.cm < c.zb ? t.k0 + c.cm : c.zb;
+        t.hz = 0;
+    } else if (b < n) {
+        const int per = c.tiles_x * c.ry, q = (b - nm) / per, e = b - nm - q * per, r = e / c.tiles_x;
+        t.ty = r < c.rl ? r : c.tiles_y - c.ry + r;
+        t.tc = e % c.tiles_x;
+        t.k0 = c.za + q * c.cy;
+        t.k1 = t.k0 + c.cy < c.zb ? t.k0 + c.cy : c.zb;
+        t.hz = 0;
+    } else {
+        const int per = c.tiles_x * c.tiles_y, e = (b - n) % per;
+        const bool low = c.za > 0 && b - n < per;
+        t.ty = e / c.tiles_x;
+        t.tc = e % c.tiles_x;
+        t.k0 = low ? 0 : c.zb;
+        t.k1 = low ? c.za : c.nz;
+        t.hz = c.layer;
+    }
+    return t;
+}
+
 struct Args {
     Grid g;
     float *out[6];          // output field set
     Cpml pm;                // psi read (hin: H set cur, e: E set ecur) and coefficients
     float *eout[3][2];      // E psi written (set ecur^1); H psi: pm.hout
-    int ta, tb, nl, nw, tiles_x, tiles_y;   // tile columns (tile_col), tiles_x = their number
-    int za, zb, cm, m;      // z chunks: m of cm planes over [za, zb), then [0, za), [zb, nz)
+    int ta, tb, nl, nw;     // tile columns (tile_col)
+    Cut cut;                // the blocks of the launch
     int zt;                 // planes of the z coefficient table
     int smem_floats;        // floats of dynamic shared memory after the barriers
     int xlo4, xhb, xbw;     // x psi: high half start, first column of the high half, box width
@@ -754,7 +801,7 @@ __device__ __forceinline__ void march_z(bool hz, bool edge, const Args &A, const
 // one kernel with the others, the larger code slowed those: 384x384x1536 1339 ->
 // 1361 us a step, and 1387 with the test of the current's planes)
 template <bool FT, int VW>
-__device__ __forceinline__ void run_block(const Args &A, const Maps &M, const TileCol T, int ty) {
+__device__ __forceinline__ void run_block(const Args &A, const Maps &M, const TileCol T, const Item it) {
     typedef Geo<VW> G;
     constexpr int TXC = G::TXC, PBOX = G::PBOX, FIELDS = G::FIELDS, CX = G::CX, CY = G::CY, CZ = G::CZ;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -768,27 +815,13 @@ __device__ __forceinline__ void run_block(const Args &A, const Maps &M, const Ti
     const int P = pm.P;
     const int tid = threadIdx.x;
     Blk B;
-    const int tile = (int)blockIdx.x;
     B.i0 = T.i0;
     B.iend = T.i0 + T.w;
-    B.j0 = ty * TY;
-    {
-        // chunk-major launch order: the middle chunks first, the two layer
-        // chunks last
-        const int c = (int)blockIdx.y;
-        if (c < A.m) {
-            B.k0 = A.za + c * A.cm;
-            B.k1 = min(A.zb, B.k0 + A.cm);
-        } else if (c == A.m && A.za > 0) {
-            B.k0 = 0;
-            B.k1 = A.za;
-        } else {
-            B.k0 = A.zb;
-            B.k1 = g.nz;
-        }
-        B.hz = P > 0 && c >= A.m;
-        B.rec = (c * A.tiles_x * A.tiles_y + tile) * TY;
-    }
+    B.j0 = it.ty * TY;
+    B.k0 = it.k0;
+    B.k1 = it.k1;
+    B.hz = it.hz != 0;
+    B.rec = (int)blockIdx.x * TY;
     B.kstart = B.k0 - 2;
     B.nplanes = B.k1 - B.k0 + 4;   // input planes k0-2 .. k1+1
     B.src_blk = A.src.active && B.i0 - 4 <= A.src.ic + A.src.L && B.i0 + TXC - 5 >= A.src.ic - A.src.L &&
@@ -920,15 +953,14 @@ __device__ __forceinline__ void run_block(const Args &A, const Maps &M, const Ti
 }
 
 __global__ void __launch_bounds__(NT, 1) k_tb2(const Args A, const __grid_constant__ Maps M) {
-    const int tile = (int)blockIdx.x;
-    const int ty = tile / A.tiles_x;
-    const TileCol T = tile_col(tile - ty * A.tiles_x, A.ta, A.tb, A.nl, A.nw, A.g.nx, false);
-    if (T.vw == 1) run_block<false, 1>(A, M, T, ty);
-    else run_block<false, 4>(A, M, T, ty);
+    const Item it = item(A.cut, (int)blockIdx.x);
+    const TileCol T = tile_col(it.tc, A.ta, A.tb, A.nl, A.nw, A.g.nx, false);
+    if (T.vw == 1) run_block<false, 1>(A, M, T, it);
+    else run_block<false, 4>(A, M, T, it);
 }
 
 __global__ void __launch_bounds__(NT, 1) k_tb2_full(const Args A, const __grid_constant__ Maps M) {
-    run_block<true, 4>(A, M, tile_col(0, 0, 0, 0, 1, A.g.nx, true), (int)blockIdx.x);
+    run_block<true, 4>(A, M, tile_col(0, 0, 0, 0, 1, A.g.nx, true), item(A.cut, (int)blockIdx.x));
 }
 
 constexpr CUtensorMapL2promotion kPromotion = CU_TENSOR_MAP_L2_PROMOTION_L2_128B;
@@ -937,7 +969,8 @@ struct HostState {
     Maps maps;
     int ta, tb, nl, nw;                        // tile columns (tile_col)
     bool full;
-    int tiles_x, tiles_y, za, zb, cm, m, zt, chunks, smem_floats;
+    int tiles_x, tiles_y, za, zb, zt, smem_floats;
+    Cut cut;
     int xlo4, xhb, xbw;
     size_t smem;
     // planes stored for the detectors and the places of their values, rebuilt
@@ -959,13 +992,6 @@ int tile_of(const HostState *st, int i, int nx) {
     return tc;
 }
 
-// chunk of plane k (the kernel's chunk decoding, inverted)
-int chunk_of(const HostState *st, int k) {
-    if (k < st->za) return st->m;
-    if (k >= st->zb) return st->m + (st->za > 0 ? 1 : 0);
-    return (k - st->za) / st->cm;
-}
-
 void free_records(HostState *st) {
     cudaFree(st->d_planes);
     cudaFree(st->d_idx);
@@ -979,8 +1005,19 @@ void free_records(HostState *st) {
 bool build_records(fdtd_ctx *h, HostState *st) {
     free_records(st);
     if (h->np == 0) return true;
-    const int tiles = st->tiles_x * st->tiles_y;
-    const int lists = tiles * st->chunks * TY;   // owned rows of blocks
+    const int lists = st->cut.blocks() * TY;   // owned rows of blocks
+    std::vector<std::vector<int>> blocks((size_t)st->tiles_x * st->tiles_y);   // of a tile
+    for (int b = 0; b < st->cut.blocks(); ++b) {
+        const Item t = item(st->cut, b);
+        blocks[t.ty * st->tiles_x + t.tc].push_back(b);
+    }
+    const auto block_of = [&](int tile, int k) {
+        for (int b : blocks[tile]) {
+            const Item t = item(st->cut, b);
+            if (k >= t.k0 && k < t.k1) return b;
+        }
+        return 0;   // the chunks of a tile cover the grid's planes
+    };
     // the six cells of each detector's readout: Ex at i-1, i; Ey at j-1, j; Ez at k-1, k
     struct Rec { int list, plane, place, slot; };
     std::vector<Rec> recs;
@@ -992,7 +1029,7 @@ bool build_records(fdtd_ctx *h, HostState *st) {
         for (int s = 0; s < 6; ++s) {
             const int ci = cell[s][0], cj = cell[s][1], ck = cell[s][2], tc = tile_of(st, ci, h->g.nx);
             const TileCol T = tile_col(tc, st->ta, st->tb, st->nl, st->nw, h->g.nx, st->full);
-            recs.push_back({(chunk_of(st, ck) * tiles + (cj / TY) * st->tiles_x + tc) * TY + cj % TY, ck,
+            recs.push_back({block_of((cj / TY) * st->tiles_x + tc, ck) * TY + cj % TY, ck,
                             cell[s][3] * 32 * T.vw + ci - (T.i0 - 4), 6 * t + s});
         }
     }
@@ -1025,33 +1062,31 @@ bool build_records(fdtd_ctx *h, HostState *st) {
 
 }  // namespace
 
+// us per plane of a block in units of 0.05, measured with a timer in the blocks of
+// seven grids: full tiles of a CPML grid, other wide tiles, narrow ones; each
+// clear of the layers, in a y layer, in a z layer, in both
+static const int kCost[3][4] = {{40, 54, 66, 108}, {24, 35, 41, 64}, {20, 24, 29, 35}};
+
+static bool y_layer(const Grid &g, int P, int ty) {
+    return P > 0 && (ty * TY - 2 <= P || ty * TY + TY + 1 >= g.ny - P);
+}
+
 // Time of a launch in units of 0.05 us: its blocks in launch order, each on the
-// SM that is free first.  A block costs (planes + 4) times its kind's time per
-// plane, in us measured with a timer in the blocks of seven grids: full tiles of
-// a CPML grid 2.0 (2.7 in a y layer, 3.3 in a z layer, 5.4 in both), other wide
-// tiles 1.2 (1.75, 2.05, 3.2), narrow ones 1.0 (1.2, 1.45, 1.75).  The launch
-// times it gives are within 12 % of the measured ones on 128 x 128 x 256,
-// 128 x 128 x 512 and 160 x 160 x 640.
-static long long launch_time(const HostState *st, const Grid &g, int P, long long m, int sms) {
-    static const int cost[3][4] = {{40, 54, 66, 108}, {24, 35, 41, 64}, {20, 24, 29, 35}};
-    const int mid = st->zb - st->za;
-    const int cm = mid > 0 ? (int)((mid + m - 1) / m) : 1, mm = mid > 0 ? (mid + cm - 1) / cm : 0;
+// SM that is free first, a block (planes + 4) times its kind's time per plane.
+// Within 12 % of the measured times on 128 x 128 x 256, 128 x 128 x 512 and
+// 160 x 160 x 640.
+static long long launch_time(const HostState *st, const Grid &g, int P, const Cut &cut, int sms) {
     std::vector<long long> free_at((size_t)sms, 0);   // a heap, the earliest first
     const auto later = [](long long x, long long y) { return x > y; };
     long long end = 0;
-    for (int c = 0; c < mm + (st->za > 0) + (st->zb < g.nz); ++c) {
-        const bool low = c == mm && st->za > 0;
-        const int planes = 4 + (c < mm ? std::min(cm, mid - c * cm) : low ? st->za : g.nz - st->zb);
-        for (int ty = 0; ty < st->tiles_y; ++ty) {
-            const bool y = P > 0 && (ty * TY - 2 <= P || ty * TY + TY + 1 >= g.ny - P);
-            for (int tc = 0; tc < st->tiles_x; ++tc) {
-                const bool wide = st->full || (tc >= st->nl && tc < st->nl + st->nw);
-                std::pop_heap(free_at.begin(), free_at.end(), later);
-                free_at.back() += (long long)planes * cost[!wide ? 2 : st->full && P > 0 ? 0 : 1][(c >= mm ? 2 : 0) + y];
-                end = std::max(end, free_at.back());
-                std::push_heap(free_at.begin(), free_at.end(), later);
-            }
-        }
+    for (int b = 0, n = cut.blocks(); b < n; ++b) {
+        const Item t = item(cut, b);
+        const bool wide = st->full || (t.tc >= st->nl && t.tc < st->nl + st->nw);
+        std::pop_heap(free_at.begin(), free_at.end(), later);
+        free_at.back() += (long long)(t.k1 - t.k0 + 4) *
+                          kCost[!wide ? 2 : st->full && P > 0 ? 0 : 1][(t.hz ? 2 : 0) + y_layer(g, P, t.ty)];
+        end = std::max(end, free_at.back());
+        std::push_heap(free_at.begin(), free_at.end(), later);
     }
     return end;
 }
@@ -1185,29 +1220,46 @@ int tb2_prepare(fdtd_ctx *h) {
     // more planes than L2 keeps, and the halo rows come from DRAM twice (measured:
     // 139 -> 147 Gcell/s on 384x384x1536 and 169 -> 181 on 640x640x2048 with
     // chunks of about 150 planes instead of 300-500; below 64 planes the
-    // warm-up planes cost more than L2 saves).  A launch of a few waves takes the
-    // chunks with the shortest launch_time, which counts the layer blocks that
-    // follow the middle ones (us a step, against the fewest waves x chunk length
-    // alone: 128x128x512 103 -> 94, 128x128x256 77 -> 57, 160x160x640 213 -> 174,
-    // 200x200x300 185 -> 158, all with 10 CPML cells);
-    // a longer one, where that makes no difference, the fewest waves x length.
+    // warm-up planes cost more than L2 saves).  The launch takes the chunks with the
+    // shortest launch_time, which counts the layer blocks that follow the middle
+    // ones and lets the tile rows of the y layers, 1.4 times as slow per plane, have
+    // shorter chunks.  us a step with 10 CPML cells, the fewest waves x chunk length
+    // alone, then with launch_time, then with chunks of their own for the y layers:
+    // 128x128x512 103, 93, 79; 128x128x256 77, 57, 51; 128x256x512 164, 162, 132;
+    // 160x160x640 213, 174, 173; 200x200x300 185, 158, 161; 384x384x768 739, 721,
+    // 684; 384x384x1536 1340, -, 1320; 640x640x2048 4040, -, 4057.
     constexpr long long CM_MAX = 160;
     const int mid = st->zb - st->za;
     const int sms = h->num_sms > 0 ? h->num_sms : 1;
     const long long tiles = (long long)st->tiles_x * st->tiles_y;
-    long long m = 0, best = -1;
+    long long best = -1;
     const long long m_lo = std::max(1LL, (mid + CM_MAX - 1) / CM_MAX);
     const long long m_hi = std::max(m_lo, (long long)(mid / 16));
-    const bool few = tiles * m_lo <= 8LL * sms;
-    if (mid > 0)
-        for (long long mm = m_lo; mm <= (few ? std::min(m_hi, m_lo + 24) : m_hi); ++mm) {
-            const long long cm = (mid + mm - 1) / mm;
-            const long long cost = few ? launch_time(st, g, P, mm, sms) : (tiles * mm + sms - 1) / sms * (cm + 7);
-            if (best < 0 || cost < best) { best = cost; m = mm; }
+    const long long tries = std::min(25LL, 30000 / (tiles * m_lo));   // 2 ms of host time at most
+    const bool few = tries > 0;   // beyond: the fewest waves x length
+    // in the tile rows of the y layers, chunks of about the other rows' time
+    Cut c{st->tiles_x, st->tiles_y, 0, 0, st->za, st->zb, g.nz, 0, 1, 0, 1, P > 0};
+    int yrows = 0, ylow = 0;
+    for (int ty = 0; ty < st->tiles_y; ++ty)
+        if (y_layer(g, P, ty)) {
+            ++yrows;
+            if (ylow == ty) ++ylow;
         }
-    st->cm = m > 0 ? (int)((mid + m - 1) / m) : 1;
-    st->m = m > 0 ? (mid + st->cm - 1) / st->cm : 0;
-    st->chunks = st->m + (st->za > 0 ? 1 : 0) + (st->zb < g.nz ? 1 : 0);
+    const int *kind = kCost[st->full && P > 0 ? 0 : 1];
+    st->cut = c;
+    if (mid > 0)
+        for (long long mm = m_lo; mm <= (few ? std::min(m_hi, m_lo + tries - 1) : m_hi); ++mm) {
+            c.cm = (int)((mid + mm - 1) / mm);
+            c.m = (mid + c.cm - 1) / c.cm;
+            for (int split = 0; split < (few && yrows > 0 ? 2 : 1); ++split) {
+                c.ry = split ? yrows : 0;
+                c.rl = split ? ylow : 0;
+                c.cy = split ? std::max(1, (c.cm + 4) * kind[0] / kind[1] - 4) : 1;
+                c.my = split ? (mid + c.cy - 1) / c.cy : 0;
+                const long long cost = few ? launch_time(st, g, P, c, sms) : (tiles * mm + sms - 1) / sms * (c.cm + 7);
+                if (best < 0 || cost < best) { best = cost; st->cut = c; }
+            }
+        }
     if (floats - G4::head_floats(st->zt) < 2 * (st->full ? bigF : big4) || floats - G1::head_floats(st->zt) < 2 * big1 ||
         cudaFuncSetAttribute(st->full ? k_tb2_full : k_tb2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st->smem) != cudaSuccess) {
         cudaGetLastError();
@@ -1259,12 +1311,7 @@ void launch_tb2(fdtd_ctx *h, cudaStream_t s) {
     a.tb = st->tb;
     a.nl = st->nl;
     a.nw = st->nw;
-    a.tiles_x = st->tiles_x;
-    a.tiles_y = st->tiles_y;
-    a.za = st->za;
-    a.zb = st->zb;
-    a.cm = st->cm;
-    a.m = st->m;
+    a.cut = st->cut;
     a.zt = st->zt;
     a.smem_floats = st->smem_floats;
     a.xlo4 = st->xlo4;
@@ -1282,7 +1329,7 @@ void launch_tb2(fdtd_ctx *h, cudaStream_t s) {
     a.planes = st->d_planes;
     a.pidx = st->d_idx;
     a.pbuf = st->d_pbuf;
-    dim3 grid(st->tiles_x * st->tiles_y, st->chunks);
+    const unsigned grid = (unsigned)st->cut.blocks();
     if (st->full) k_tb2_full<<<grid, NT, st->smem, s>>>(a, st->maps);
     else k_tb2<<<grid, NT, st->smem, s>>>(a, st->maps);
 }
