@@ -60,6 +60,13 @@ void release(fdtd_ctx *h) {
     delete h;
 }
 
+// The detectors' records of the paths that keep some (here, not in the first
+// step that needs them: the stream may be captured then).
+void new_probes(fdtd_ctx *h) {
+    res_set_probes(h);
+    if (h->kernel == 2 && h->tb2) tb2_ready(h);
+}
+
 // Fewest cells for which the two-step path is the default.  Measured, us a step,
 // path 1 and path 2: PEC grids too large for the resident path 20.7, 18.6 (100^3),
 // 31.5, 21.6 (150x100x100), 87.6, 44 (128x128x512); CPML grids of one tile column
@@ -119,10 +126,18 @@ constexpr int RES_MIN_STEPS = 2;
 // n steps of the handle's selected path, issued on `st` (the handle's own
 // stream for fdtd_step; a batch's stream when the batch steps it alone).
 int fdtd_step_on(fdtd_ctx *h, int n, cudaStream_t st) {
+    // a small grid's runs and two-step passes are not captured into a graph, where
+    // an even number of single steps leaves the state in the set it began with
+    bool runs = h->res || h->two_step_small;
+    if (runs) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        runs = cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+        if (!runs) cudaGetLastError();
+    }
     for (int s = 0; s < n;) {
         int adv = 1;
         // runs of steps of a small grid in one launch, up to the next watchdog check
-        if (h->kernel == 1 && n - s >= RES_MIN_STEPS && res_ready(h, st)) {
+        if (runs && h->kernel == 1 && n - s >= RES_MIN_STEPS && res_ready(h)) {
             int m = n - s < res_steps() ? n - s : res_steps();
             if (h->watch_every > 0) {
                 const long long next = h->watch_every - h->steps % h->watch_every;
@@ -138,7 +153,7 @@ int fdtd_step_on(fdtd_ctx *h, int n, cudaStream_t st) {
             }
             res_release(h);   // refused: the one-step path from here on
         }
-        if (h->kernel == 2 && n - s >= 2 && tb2_ready(h)) {
+        if (h->kernel == 2 && n - s >= 2 && (runs || !h->two_step_small) && tb2_ready(h)) {
             // two steps in one pass; the detectors of both from its records
             timed_launch(h, st, [](const fdtd_ctx *c, cudaStream_t q) { launch_tb2(const_cast<fdtd_ctx *>(c), q); });
             if (h->np > 0) { launch_tb2_probes(h, st); h->launches++; }
@@ -292,7 +307,10 @@ int fdtd_create(fdtd_t *out, int nx, int ny, int nz, double dx, double dt, doubl
         h->kernel = 1;
         res_prepare(h);
     }
-    if (!h->res && (long long)nx * ny * nz >= two_step_min_cells(h) && tb2_prepare(h) == FDTD_OK) h->kernel = 2;
+    if (!h->res && (long long)nx * ny * nz >= two_step_min_cells(h) && tb2_prepare(h) == FDTD_OK) {
+        h->kernel = 2;
+        h->two_step_small = (long long)nx * ny * nz < FDTD_TWO_STEP_MIN_CELLS;
+    }
     cudaGetLastError();
     *out = h;
     return FDTD_OK;
@@ -373,8 +391,10 @@ int fdtd_set_probes(fdtd_t h, const double *xyz, int n, int max_steps) {
     h->np = 0; h->max_steps = max_steps;
     h->probe_ver++;
     h->h_ijk.clear();
-    res_set_probes(h);
-    if (n == 0) return FDTD_OK;
+    if (n == 0) {
+        new_probes(h);
+        return FDTD_OK;
+    }
     size_t tb = sizeof(float) * 2 * (size_t)n * (size_t)(max_steps > 0 ? max_steps : 1);
     if (cudaMalloc(&h->d_ijk, sizeof(int) * 3 * n) != cudaSuccess ||
         cudaMalloc(&h->d_cxy, sizeof(float) * 2 * n) != cudaSuccess ||
@@ -387,7 +407,7 @@ int fdtd_set_probes(fdtd_t h, const double *xyz, int n, int max_steps) {
     TRY(h, cudaMemset(h->d_trace, 0, tb));
     h->np = n;
     h->h_ijk = ijk;
-    res_set_probes(h);
+    new_probes(h);
     return FDTD_OK;
 }
 
@@ -645,6 +665,8 @@ int fdtd_set_kernel(fdtd_t h, int which) {
         if (rc != FDTD_OK) return rc == FDTD_ERR_CUDA ? FDTD_ERR_CUDA : FDTD_ERR_ARG;
     }
     h->kernel = which;
+    h->two_step_small = false;
+    if (which == 2) tb2_ready(h);
     return FDTD_OK;
 }
 

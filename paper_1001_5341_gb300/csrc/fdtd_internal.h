@@ -148,6 +148,7 @@ struct fdtd_ctx {
     const float *aE[3], *bE[3], *aH[3], *bH[3];
     int kernel;               // field-update path: 0 unfused sweeps, 1 vector tile,
                               // 2 two steps per pass (vector tile for a last odd step)
+    bool two_step_small;      // path 2 by default on a grid below FDTD_TWO_STEP_MIN_CELLS
     void *vtile;              // host state of the vector-tile path
     void *tb2;                // host state of the two-step path
     void *res;                // host state of the resident path (null: not for this grid)
@@ -228,7 +229,7 @@ bool tb2_ready(fdtd_ctx *h);
 void res_prepare(fdtd_ctx *h);
 void res_release(fdtd_ctx *h);
 void res_set_probes(fdtd_ctx *h);                    // after the detectors changed
-bool res_ready(fdtd_ctx *h, cudaStream_t s);
+bool res_ready(const fdtd_ctx *h);
 int res_steps();                                     // most steps per launch
 bool launch_res(fdtd_ctx *h, int n, cudaStream_t s); // advances h->cur and h->steps
 // detector slots steps .. steps + n - 1 from records [n][np][6] of E (kernels_basic.cu)

@@ -654,18 +654,12 @@ void res_release(fdtd_ctx *h) {
     h->res = nullptr;
 }
 
-// Whether the resident path takes the handle's next steps on stream s.  Not
-// while launches are timed (those are single steps) and not into a graph: a
-// replay would find its exchange tags already there.
-bool res_ready(fdtd_ctx *h, cudaStream_t s) {
-    ResState *st = static_cast<ResState *>(h->res);
-    if (!st || h->timing.on) return false;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-        cudaGetLastError();
-        return false;
-    }
-    return st->probes_ok;
+// Whether the resident path takes the handle's next steps: not while launches
+// are timed (those are single steps).  The caller leaves it out while the stream
+// is captured: a replay would find its exchange tags already there.
+bool res_ready(const fdtd_ctx *h) {
+    const ResState *st = static_cast<const ResState *>(h->res);
+    return st && !h->timing.on && st->probes_ok;
 }
 
 void res_set_probes(fdtd_ctx *h) {

@@ -1235,8 +1235,11 @@ int tb2_prepare(fdtd_ctx *h) {
     long long best = -1;
     const long long m_lo = std::max(1LL, (mid + CM_MAX - 1) / CM_MAX);
     const long long m_hi = std::max(m_lo, (long long)(mid / 16));
-    const long long tries = std::min(25LL, 30000 / (tiles * m_lo));   // 2 ms of host time at most
-    const bool few = tries > 0;   // beyond: the fewest waves x length
+    // blocks scheduled over all cuts that are tried, about half a millisecond of host
+    // time; beyond, the fewest waves x length
+    constexpr long long MAX_WORK = 16000;
+    long long work = 0;
+    const bool few = tiles * m_lo <= MAX_WORK;
     // in the tile rows of the y layers, chunks of about the other rows' time
     Cut c{st->tiles_x, st->tiles_y, 0, 0, st->za, st->zb, g.nz, 0, 1, 0, 1, P > 0};
     int yrows = 0, ylow = 0;
@@ -1248,7 +1251,7 @@ int tb2_prepare(fdtd_ctx *h) {
     const int *kind = kCost[st->full && P > 0 ? 0 : 1];
     st->cut = c;
     if (mid > 0)
-        for (long long mm = m_lo; mm <= (few ? std::min(m_hi, m_lo + tries - 1) : m_hi); ++mm) {
+        for (long long mm = m_lo; mm <= m_hi && work <= MAX_WORK; ++mm) {
             c.cm = (int)((mid + mm - 1) / mm);
             c.m = (mid + c.cm - 1) / c.cm;
             for (int split = 0; split < (few && yrows > 0 ? 2 : 1); ++split) {
@@ -1256,6 +1259,7 @@ int tb2_prepare(fdtd_ctx *h) {
                 c.rl = split ? ylow : 0;
                 c.cy = split ? std::max(1, (c.cm + 4) * kind[0] / kind[1] - 4) : 1;
                 c.my = split ? (mid + c.cy - 1) / c.cy : 0;
+                if (few) work += c.blocks();
                 const long long cost = few ? launch_time(st, g, P, c, sms) : (tiles * mm + sms - 1) / sms * (c.cm + 7);
                 if (best < 0 || cost < best) { best = cost; st->cut = c; }
             }

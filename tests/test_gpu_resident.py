@@ -83,3 +83,40 @@ def test_resident_handles_side_by_side(fd):
     assert max(launches[:3]) < steps < launches[3]
     for t in traces:
         assert np.abs(t).max() > 0 and np.array_equal(t, np.repeat(traces[0], len(t), 0))
+
+
+@pytest.mark.parametrize("shape,npml", [((30, 33, 40), 0), ((130, 20, 12), 0), ((128, 128, 160), 8)])
+def test_captured_steps_replay(fd, shape, npml):
+    """An even number of steps captured into a graph (no shower, no detectors)
+    replays as that many further steps, on every grid whose default steps go
+    several to a launch."""
+    import torch
+    nx, ny, nz = shape
+    dx = 0.02
+    dt = W.courant_dt(dx, W.EPS_R_ICE)
+    b = fd.FDTD_CPML if npml else fd.FDTD_PEC
+    start = np.random.default_rng(5).standard_normal((nz + 1, ny + 1, nx + 1)).astype(np.float32)
+    start[:npml + 2] = start[-npml - 2:] = 0
+    start[:, :npml + 2] = start[:, -npml - 2:] = 0
+    start[:, :, :npml + 2] = start[:, :, -npml - 2:] = 0
+    st = torch.cuda.Stream()
+    sim = fd.Simulation(nx, ny, nz, dx, dt, W.EPS_R_ICE, b, npml, stream=st)
+    ref = fd.Simulation(nx, ny, nz, dx, dt, W.EPS_R_ICE, b, npml)
+    for s in (sim, ref):
+        s.set_field("Ez", start)
+        s.sync()
+    ref.set_kernel(1)
+    g = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, stream=st):
+        sim.step(4)
+    for _ in range(3):
+        g.replay()
+    torch.cuda.synchronize()
+    for _ in range(12):
+        ref.step(1)
+    for c in ("Ex", "Ez", "Hy"):
+        want = ref.field(c)
+        assert np.abs(want).max() > 0 and np.array_equal(sim.field(c), want)
+    sim.close()
+    ref.close()
