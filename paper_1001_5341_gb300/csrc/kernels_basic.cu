@@ -17,6 +17,7 @@
 
 #include "cell_update.cuh"
 #include "fdtd_internal.h"
+#include "launch_chain.cuh"
 #include "source_term.cuh"
 
 namespace fdtd {
@@ -103,8 +104,10 @@ __global__ void k_probes(Grid g, const float *__restrict__ E, Probes p, long lon
 
 // After a two-step pass: slot n from the rows of E^{n+1} that the pass stored
 // (pos: the places of the six values per detector), slot n+1 from E^{n+2} (set cur^1).
-__global__ void k_probes2(Grid g, const float *__restrict__ E, Probes p, long long slot,
-                          const float *__restrict__ rec, const int *__restrict__ pos) {
+__global__ void k_probes2(Grid g, const float *E, Probes p, long long slot,
+                          const float *rec, const int *__restrict__ pos) {
+    release_next_launch();
+    after_last_launch();
     int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= p.n) return;
     float v[6];
@@ -137,7 +140,8 @@ void launch_tb2_probes(fdtd_ctx *h, cudaStream_t s) {
     const int *pos = nullptr;
     const float *rec = tb2_probe_values(h, &pos);
     if (!rec) return;
-    k_probes2<<<(h->np + 127) / 128, 128, 0, s>>>(h->g, h->fields[h->cur ^ 1], p, h->steps, rec, pos);
+    launch_after(h->P == 0, k_probes2, dim3((h->np + 127) / 128), dim3(128), 0, s, h->g,
+                 (const float *)h->fields[h->cur ^ 1], p, h->steps, rec, pos);
 }
 
 // Watchdog of the step path: block (x, y) scans plane k = min(y * stride,
