@@ -1079,17 +1079,20 @@ static bool y_layer(const Grid &g, int P, int ty) {
 // Within 12 % of the measured times on 128 x 128 x 256, 128 x 128 x 512 and
 // 160 x 160 x 640.
 static long long launch_time(const HostState *st, const Grid &g, int P, const Cut &cut, int sms) {
-    std::vector<long long> free_at((size_t)sms, 0);   // a heap, the earliest first
+    constexpr int MAX_SMS = 1024;
+    long long free_at[MAX_SMS] = {};   // a heap, the earliest first
+    sms = std::min(sms, MAX_SMS);
+    long long *const last = free_at + sms - 1;
     const auto later = [](long long x, long long y) { return x > y; };
     long long end = 0;
     for (int b = 0, n = cut.blocks(); b < n; ++b) {
         const Item t = item(cut, b);
         const bool wide = st->full || (t.tc >= st->nl && t.tc < st->nl + st->nw);
-        std::pop_heap(free_at.begin(), free_at.end(), later);
-        free_at.back() += (long long)(t.k1 - t.k0 + 4) *
+        std::pop_heap(free_at, free_at + sms, later);
+        *last += (long long)(t.k1 - t.k0 + 4) *
                           kCost[!wide ? 2 : st->full && P > 0 ? 0 : 1][(t.hz ? 2 : 0) + y_layer(g, P, t.ty)];
-        end = std::max(end, free_at.back());
-        std::push_heap(free_at.begin(), free_at.end(), later);
+        end = std::max(end, *last);
+        std::push_heap(free_at, free_at + sms, later);
     }
     return end;
 }
